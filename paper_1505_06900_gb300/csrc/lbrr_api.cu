@@ -23,6 +23,10 @@ struct lb_ctx {
   int device = 0;
   size_t elem = 4;         // bytes per stored population
   void *f = nullptr;       // population store, q * n elements
+  void *run = nullptr;     // scratch of the kernels for runs of updates, allocated on first
+                           // use; between calls the state is always in f
+  bool run_off = false;    // it does not fit: update by update
+  int sms = 0;                 // SMs of the device
   int red_blocks = 0;          // partial-sum blocks: kRedBlocksPerSm x the device's SMs
   double *partials = nullptr;  // reduction scratch, red_blocks * kRedValues doubles
   double *dout = nullptr;      // reduction result, kRedValues doubles
@@ -137,6 +141,8 @@ int free_all(lb_ctx *c) {
   if (c->capture) cudaStreamDestroy(c->capture);
   c->capture = nullptr;
   if (c->f) cudaFree(c->f);
+  if (c->run) cudaFree(c->run);
+  c->run = nullptr;
   if (c->partials) cudaFree(c->partials);
   if (c->dout) cudaFree(c->dout);
   if (c->status) cudaFree(c->status);
@@ -262,6 +268,7 @@ int lb_create_ex(lb_ctx **out, const lb_options *opt) {
     delete c;
     return fail(nullptr, LB_ECUDA, "cannot query the SM count: %s", cudaGetErrorString(e));
   }
+  c->sms = sms;
   c->red_blocks = lbrr::kRedBlocksPerSm * sms;
   const size_t bytes = c->elem * (size_t)c->q * (size_t)n;
   e = cudaMalloc(&c->f, bytes);
@@ -360,6 +367,26 @@ cudaGraphExec_t step_graph(lb_ctx *c, float om1) {
   return c->graph[p];
 }
 
+// The scratch for runs of updates, allocated on first use where it takes at
+// most a quarter of the device's free memory (the context works without it,
+// one update at a time). The allocation must not disturb a stream capture
+// that another thread or stream has under way.
+bool ensure_run(lb_ctx *c, size_t bytes) {
+  if (c->run || c->run_off) return c->run != nullptr;
+  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+  cudaThreadExchangeStreamCaptureMode(&mode);
+  size_t free_b = 0, total_b = 0;
+  cudaError_t e = cudaMemGetInfo(&free_b, &total_b);
+  if (e == cudaSuccess && bytes <= free_b / 4) e = cudaMalloc(&c->run, bytes);
+  cudaThreadExchangeStreamCaptureMode(&mode);
+  if (e != cudaSuccess) {
+    cudaGetLastError();
+    c->run = nullptr;
+  }
+  c->run_off = !c->run;
+  return c->run != nullptr;
+}
+
 }  // namespace
 
 int lb_step(lb_ctx *c, int n) {
@@ -375,6 +402,16 @@ int lb_step(lb_ctx *c, int n) {
   const bool capturing = cudaStreamIsCapturing(c->stream, &cs) != cudaSuccess ||
                          cs != cudaStreamCaptureStatusNone;
   if (capturing) cudaGetLastError();
+  if (!c->closure && !capturing &&
+      lbrr::moment_run_supported(c->q, c->storage, c->collision, c->g, n, c->sms) &&
+      ensure_run(c, lbrr::moment_run_bytes(c->g))) {
+    cudaError_t e = lbrr::launch_moment_run(c->q, c->collision, c->f, c->run, c->g, om1, c->parity,
+                                            n, c->sms, c->stream);
+    if (e != cudaSuccess) return cuda_fail(c, e, "step launch");
+    c->parity = (c->parity + n) & 1;
+    c->steps += n;
+    return LB_OK;
+  }
   while (!c->closure && !capturing && n >= kGraphSteps) {
     cudaGraphExec_t ge = step_graph(c, om1);
     if (!ge) break;

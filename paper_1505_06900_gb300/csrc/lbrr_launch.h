@@ -21,6 +21,13 @@ constexpr int kRedValues = 5;      // partial sums per block (mass, momentum x3,
 cudaError_t launch_step(int q, int storage, int model, void *f, const Grid &g, float om1,
                         int parity, int *status, cudaStream_t st);
 
+// `steps` >= 1 updates of the periodic 3-D FP32 store `f` of the given parity on
+// its moments (lbrr_run3.cu), through scratch of moment_run_bytes.
+bool moment_run_supported(int q, int storage, int model, const Grid &g, int steps, int sms);
+size_t moment_run_bytes(const Grid &g);
+cudaError_t launch_moment_run(int q, int model, void *f, void *scratch, const Grid &g, float om1,
+                              int parity, int steps, int sms, cudaStream_t st);
+
 // The one-thread-per-cell kernel of launch_step (lbrr_step.cu), for any grid
 // without walls and any storage.
 cudaError_t launch_step_cell(int q, int storage, int model, void *f, const Grid &g, float om1,
