@@ -26,6 +26,7 @@ struct lb_ctx {
   void *run = nullptr;     // scratch of the kernels for runs of updates, allocated on first
                            // use; between calls the state is always in f
   bool run_off = false;    // it does not fit: update by update
+  lbrr::Run2Plans run2;    // D2Q9: the tiles of a run's passes, set on first use
   int sms = 0;                 // SMs of the device
   int red_blocks = 0;          // partial-sum blocks: kRedBlocksPerSm x the device's SMs
   double *partials = nullptr;  // reduction scratch, red_blocks * kRedValues doubles
@@ -407,6 +408,17 @@ int lb_step(lb_ctx *c, int n) {
       ensure_run(c, lbrr::moment_run_bytes(c->g))) {
     cudaError_t e = lbrr::launch_moment_run(c->q, c->collision, c->f, c->run, c->g, om1, c->parity,
                                             n, c->sms, c->stream);
+    if (e != cudaSuccess) return cuda_fail(c, e, "step launch");
+    c->parity = (c->parity + n) & 1;
+    c->steps += n;
+    return LB_OK;
+  }
+  if (!c->closure && !capturing &&
+      lbrr::moment_run2_supported(c->q, c->storage, c->collision, c->g, n) &&
+      ensure_run(c, lbrr::moment_run2_bytes(c->g))) {
+    if (!c->run2.ready) lbrr::plan_moment_run2(c->g, c->sms, &c->run2);
+    cudaError_t e = lbrr::launch_moment_run2(c->f, c->run, c->g, om1, c->parity, n, c->run2,
+                                             c->stream);
     if (e != cudaSuccess) return cuda_fail(c, e, "step launch");
     c->parity = (c->parity + n) & 1;
     c->steps += n;

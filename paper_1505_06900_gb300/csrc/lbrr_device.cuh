@@ -243,9 +243,8 @@ __device__ __forceinline__ void synth1(float c0, float c1, float c2, float &om, 
   } else {
     const float q = fmaf(c0, kCs2, c2);
     oz = c0 - q;
-    const float h = 0.5f * q;  // 0.5 (q +- c1): exact halves, rounded once
-    op = fmaf(0.5f, c1, h);
-    om = fmaf(-0.5f, c1, h);
+    op = 0.5f * (q + c1);
+    om = 0.5f * (q - c1);
   }
 }
 

@@ -28,6 +28,35 @@ size_t moment_run_bytes(const Grid &g);
 cudaError_t launch_moment_run(int q, int model, void *f, void *scratch, const Grid &g, float om1,
                               int parity, int steps, int sms, cudaStream_t st);
 
+// The same for a periodic D2Q9 FP32 store (lbrr_run2.cu).
+constexpr int kRun2Units = 12;  // updates a pass at most
+struct Plan2 {
+  int tiles_x, tiles_y, ox, oy;  // tiles of ox x oy cells
+  int ex, cells;                 // a tile with its halo: row length and cells
+  double us;                     // estimated time of the pass (negative: none fits)
+};
+// The same for the kernel that walks down the rows (lbrr_run2m.cu).
+struct PlanM {
+  int ex;                // cells of a row a block advances
+  int tiles_x, ox, seg;  // columns of ox cells, segments of seg rows
+  int blocks;
+  double us;
+};
+struct Run2Plans {
+  bool ready = false;
+  Plan2 tile[kRun2Units + 1];  // by the number of updates
+  PlanM march[kRun2Units + 1];
+};
+PlanM plan_march(const Grid &g, int units, int sms);
+// kind 0: moments a to moments b, 1: the store f to b, 2: a to f.
+cudaError_t launch_march(int kind, float *f, const float *a, float *b, const Grid &g, float om1,
+                         const PlanM &q, int units, int parity, cudaStream_t st);
+bool moment_run2_supported(int q, int storage, int model, const Grid &g, int steps);
+size_t moment_run2_bytes(const Grid &g);
+void plan_moment_run2(const Grid &g, int sms, Run2Plans *plans);
+cudaError_t launch_moment_run2(void *f, void *scratch, const Grid &g, float om1,
+                               int parity, int steps, const Run2Plans &plans, cudaStream_t st);
+
 // The one-thread-per-cell kernel of launch_step (lbrr_step.cu), for any grid
 // without walls and any storage.
 cudaError_t launch_step_cell(int q, int storage, int model, void *f, const Grid &g, float om1,

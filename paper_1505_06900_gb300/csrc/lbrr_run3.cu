@@ -11,7 +11,7 @@
 // the layout the same number of single updates would leave. Every value is
 // computed by the operations of the single updates in their order (the
 // moments' sums over x, y, then z are split by z component), so the result is
-// theirs bit for bit.
+// theirs bit for bit unless something underflows.
 #include "lbrr_launch.h"
 
 namespace lbrr {
@@ -452,7 +452,7 @@ cudaError_t run_t(float *f, float *m0, float *m1, const Grid &g, float om1, int 
 // bytes a cell at the copy rate), its first and last passes cost 296 / 216 or
 // 232 / 152, and an update between them 0.52 (D3Q27) or 0.60 (D3Q19) of the
 // cells its plane iterations could hold, which is what the kernel measures at
-// 256^3 and 512^3; 0.08 and 0.10 are added on the safe side. Measured on both
+// 256^3 and 512^3; 0.10 and 0.14 are added on the safe side. Measured on both
 // sides of the lines (microseconds an update, single / moments): 96x60x64
 // 10.5 / 15.3, 640x130x9 19.3 / 24.3, 128^3 70.3 / 51.4 (40 updates) and 72.7 /
 // 68.3 (3), 250x151x101 131 / 94.8; D3Q19 128^3 50.8 / 52.0 (6 updates),
@@ -463,7 +463,7 @@ bool moment_run_supported(int q, int storage, int model, const Grid &g, int step
     return false;
   const int ty = q == 27 ? Tile<27>::TY : Tile<19>::TY;
   const double held = (double)plan_of(ty, g, sms).planes * sms * ty * kTX;
-  const double ends = q == 27 ? 296.0 / 216.0 : 232.0 / 152.0, rate = q == 27 ? 0.60 : 0.70;
+  const double ends = q == 27 ? 296.0 / 216.0 : 232.0 / 152.0, rate = q == 27 ? 0.62 : 0.74;
   return ends * (double)g.n + (steps - 1) * rate * held < (double)steps * (double)g.n;
 }
 size_t moment_run_bytes(const Grid &g) { return 2 * sizeof(float) * (size_t)plane_floats(g) * g.nz; }

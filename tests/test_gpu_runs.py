@@ -1,11 +1,12 @@
-"""Runs of updates on the moments (lb_step(n) of periodic 3-D FP32 grids large
-enough for it) against the same number of single updates.
+"""Runs of updates on the moments (lb_step(n) of FP32 grids) against the same
+number of single updates.
 
 Both carry out the same FP32 operations in the same order, so the stores agree
-bit for bit; no tolerance is needed. Shapes: partial tiles in x (also rows of
-fewer cells than a tile), in y and in z segments, both lattices, both
+bit for bit; no tolerance is needed. 3-D shapes: partial tiles in x (also rows
+of fewer cells than a tile), in y and in z segments, both lattices, both
 regularized models, runs from and to either parity, and the fewest updates a
-run takes over.
+run takes over. 2-D shapes: halos wider than the grid, each block shape of the
+tile kernel and the row-streaming kernel.
 """
 import numpy as np
 import pytest
@@ -31,7 +32,7 @@ def _state(s):
 
 @pytest.mark.parametrize("lattice,shape,steps", [
     (B.D3Q27, (250, 151, 101), 5), (B.D3Q27, (31, 200, 200), 4), (B.D3Q27, (640, 130, 16), 6),
-    (B.D3Q27, (97, 118, 120), 9), (B.D3Q19, (160, 145, 130), 16), (B.D3Q19, (62, 287, 201), 12),
+    (B.D3Q27, (97, 118, 120), 20), (B.D3Q19, (150, 200, 180), 16), (B.D3Q19, (62, 287, 201), 12),
 ])
 @pytest.mark.parametrize("collision", [B.COLLIDE_RR, B.COLLIDE_REG2])
 @pytest.mark.parametrize("first", [0, 1])
@@ -55,6 +56,35 @@ def test_runs_equal_single_updates(lattice, shape, steps, collision, first):
         a.step(1)  # and the store goes on from there
         b.step(1)
         assert torch.equal(_state(a)[0], _state(b)[0])
+
+
+@pytest.mark.parametrize("shape,steps", [
+    ((1, 1), 6), ((5, 3), 20), ((4, 9), 21), ((128, 128), 50), ((100, 37), 23), ((37, 100), 24),
+    ((64, 4000), 9), ((251, 251), 40), ((300, 200), 4), ((701, 500), 13), ((1001, 1001), 21),
+    ((1900, 1300), 31), ((2300, 1700), 6), ((1400, 3000), 17),
+])
+@pytest.mark.parametrize("first", [0, 1])
+def test_flat_runs_equal_single_updates(shape, steps, first):
+    with B.Solver(B.D2Q9, (*shape, 1), 0.61) as a, B.Solver(B.D2Q9, (*shape, 1), 0.61) as b:
+        for s in (a, b):
+            _init(s, 7)
+            for _ in range(first):
+                s.step(1)
+        free = torch.cuda.mem_get_info()[0]
+        a.step(steps)
+        scratch = free - torch.cuda.mem_get_info()[0]
+        if a.n > 1 << 20:
+            assert scratch >= 48 * a.n, "the run was expected to work on the moments"
+        for _ in range(steps):
+            b.step(1)
+        (fa, pa), (fb, pb) = _state(a), _state(b)
+        assert pa == pb == (first + steps) % 2
+        assert torch.equal(fa, fb)
+        a.step(7)
+        for _ in range(7):
+            b.step(1)
+        assert torch.equal(_state(a)[0], _state(b)[0])
+        assert a.info()["steps"] == b.info()["steps"]
 
 
 def test_run_at_rest_and_uniform_flow():
