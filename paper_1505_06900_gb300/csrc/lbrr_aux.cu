@@ -248,54 +248,190 @@ __global__ void __launch_bounds__(kRedThreads)
   }
 }
 
-// 0.5 |curl u|^2 per cell with periodic central differences.
+// 0.5 |curl u|^2 per cell. FP64 arithmetic runs at a 64th of the FP32 rate on
+// this GPU and bounded this kernel (991 us for 256^3, whose field is read in
+// 40), so a component of the curl is formed as an unevaluated sum of two
+// floats by error-free transformations (Knuth's sum, an FMA for the square;
+// relative error below 2^-44), summed the same way over up to kCurlFlush cells,
+// and only that sum goes to FP64, between loops. A component whose square
+// would leave the range where its low part is an FP32 number, and the nodes on
+// walls, take FP64. With a cell to a thread that took 227 us, waiting for
+// twelve scalar loads; with four cells of a row, which the float4 rows of
+// nx % 4 == 0 allow, 106 us.
+constexpr int kCurlFlush = 64;
+struct Float2Sum {
+  float s = 0.f, e = 0.f;
+  __device__ __forceinline__ void add(float v, float err) {
+    const float t = s + v, b = t - s;
+    e += ((s - (t - b)) + (v - b)) + err;
+    s = t;
+  }
+};
+__device__ __forceinline__ void two_diff(float a, float b, float &s, float &e) {
+  s = a - b;
+  const float v = s - a;
+  e = (a - (s - v)) - (b + v);
+}
+
+// FP64 work stays out of line and out of the loop's registers: as part of the
+// loop its operations were issued for every cell, predicated off (748 us).
+__device__ __noinline__ void add_wide(double *acc, float up, float um, float vp, float vm) {
+  const double w = ((double)up - (double)um) - ((double)vp - (double)vm);
+  *acc += 0.125 * w * w;
+}
+// A node on walls: second-order one-sided differences on the wall planes of a
+// walled axis, and half the weight for every plane it lies on.
 template <int D>
+__device__ __noinline__ void add_wall_node(double *acc, const float *__restrict__ u, const Grid &g,
+                                           int x, int y, int z) {
+  const int p[3] = {x, y, z}, dims[3] = {g.nx, g.ny, g.nz};
+  auto diff = [&](int comp, int axis) -> double {
+    int q[3] = {p[0], p[1], p[2]};
+    auto at = [&](int k) -> double {
+      q[axis] = k;
+      return (double)u[comp * g.n + ((long long)q[2] * g.ny + q[1]) * g.nx + q[0]];
+    };
+    const int a = p[axis], m = dims[axis];
+    if ((g.walls >> axis) & 1) {
+      if (a == 0) {
+        const double u0 = at(0), u1 = at(1), u2 = at(2);
+        return 0.5 * (-3.0 * u0 + 4.0 * u1 - u2);
+      }
+      if (a == m - 1) {
+        const double u0 = at(m - 1), u1 = at(m - 2), u2 = at(m - 3);
+        return 0.5 * (3.0 * u0 - 4.0 * u1 + u2);
+      }
+    }
+    const double up = at(a + 1 == m ? 0 : a + 1);
+    const double um = at(a == 0 ? m - 1 : a - 1);
+    return 0.5 * (up - um);
+  };
+  double wgt = 1.0;
+  for (int a = 0; a < D; ++a)
+    if (((g.walls >> a) & 1) && (p[a] == 0 || p[a] == dims[a] - 1)) wgt *= 0.5;
+  const double wz = diff(1, 0) - diff(0, 1);
+  double wx = 0.0, wy = 0.0;
+  if (D == 3) {
+    wx = diff(2, 1) - diff(1, 2);
+    wy = diff(0, 2) - diff(2, 0);
+  }
+  *acc += wgt * 0.5 * (wx * wx + wy * wy + wz * wz);
+}
+
+// A thread takes V cells of a row; a block's item is a stretch of a row or, of
+// rows shorter than that, as many whole rows as the block has threads for.
+template <int D, int V>
 __global__ void __launch_bounds__(kRedThreads)
     enstrophy_partial_kernel(const float *__restrict__ u, const Grid g,
                              double *__restrict__ partials) {
-  double acc[1] = {0.0};
-  const long long n = g.n;
-  const long long stride = (long long)gridDim.x * kRedThreads;
-  for (long long cell = (long long)blockIdx.x * kRedThreads + threadIdx.x; cell < n;
-       cell += stride) {
-    int x, y, z;
-    cell_coords(cell, g, x, y, z);
-    const int p[3] = {x, y, z}, dims[3] = {g.nx, g.ny, g.nz};
-    // d u_comp / d x_axis: central differences (periodic across periodic
-    // faces); second-order one-sided on the wall planes of a walled axis
-    auto diff = [&](int comp, int axis) -> double {
-      int q[3] = {p[0], p[1], p[2]};
-      auto at = [&](int k) -> double {
-        q[axis] = k;
-        return (double)u[comp * n + ((long long)q[2] * g.ny + q[1]) * g.nx + q[0]];
-      };
-      const int a = p[axis], m = dims[axis];
-      if ((g.walls >> axis) & 1) {
-        if (a == 0) {
-          const double u0 = at(0), u1 = at(1), u2 = at(2);
-          return 0.5 * (-3.0 * u0 + 4.0 * u1 - u2);
-        }
-        if (a == m - 1) {
-          const double u0 = at(m - 1), u1 = at(m - 2), u2 = at(m - 3);
-          return 0.5 * (3.0 * u0 - 4.0 * u1 + u2);
-        }
+  double acc[1] = {0.0}, rare = 0.0;
+  const long long n = g.n, rows = (long long)g.ny * g.nz, slab = (long long)g.nx * g.ny;
+  const int row_threads = g.nx / V;
+  const int per_item = row_threads < kRedThreads ? kRedThreads / row_threads : 1;
+  const int ty = per_item > 1 ? threadIdx.x / row_threads : 0;
+  const int tx = threadIdx.x - ty * row_threads;  // one row an item: threadIdx.x
+  const int chunks = per_item > 1 ? 1 : (row_threads + kRedThreads - 1) / kRedThreads;
+  const long long items = (rows + per_item - 1) / per_item * chunks;
+  const long long batch = (long long)(kCurlFlush / V) * gridDim.x;
+  for (long long first = blockIdx.x; first < items; first += batch) {
+    Float2Sum part;
+    const long long end = min(items, first + batch);
+#pragma unroll 1
+    for (long long it = first; it < end; it += gridDim.x) {
+      long long r;
+      int x = tx, y, z;
+      if (items <= 0x7FFFFFFFLL && rows <= 0x7FFFFFFFLL) {  // 32-bit divisions
+        const unsigned i = (unsigned)it, c = i / (unsigned)chunks;
+        x += (int)(i - c * (unsigned)chunks) * kRedThreads;
+        const unsigned rr = c * (unsigned)per_item + (unsigned)ty;
+        z = (int)(rr / (unsigned)g.ny);
+        y = (int)(rr - (unsigned)z * (unsigned)g.ny);
+        r = rr;
+      } else {
+        r = it / chunks;
+        x += (int)(it - r * chunks) * kRedThreads;
+        r = r * per_item + ty;
+        z = (int)(r / g.ny);
+        y = (int)(r - (long long)z * g.ny);
       }
-      const double up = at(a + 1 == m ? 0 : a + 1);
-      const double um = at(a == 0 ? m - 1 : a - 1);
-      return 0.5 * (up - um);
-    };
-    double wgt = 1.0;
+      if (x >= row_threads || ty >= per_item || r >= rows) continue;
+      x *= V;
+      const bool plane = g.walls && (((g.walls & 2) && (y == 0 || y == g.ny - 1)) ||
+                                     (D == 3 && (g.walls & 4) && (z == 0 || z == g.nz - 1)));
+      // the rows of the neighbours along y and z
+      const float *row = u + r * g.nx + x;
+      const long long yp = (long long)(y + 1 == g.ny ? 1 - g.ny : 1) * g.nx;
+      const long long ym = (long long)(y == 0 ? g.ny - 1 : -1) * g.nx;
+      const long long zp = (z + 1 == g.nz ? 1 - g.nz : 1) * slab;
+      const long long zm = (z == 0 ? g.nz - 1 : -1) * slab;
+      auto load = [&](float (&v)[V], int comp, long long off) {
+        const float *q = row + comp * n + off;
+        if constexpr (V == 4) {
+          const float4 t = *reinterpret_cast<const float4 *>(q);
+          v[0] = t.x, v[1] = t.y, v[2] = t.z, v[3] = t.w;
+        } else {
+          v[0] = *q;
+        }
+      };
+      // the cells' neighbours along x
+      auto load_x = [&](float (&p)[V], float (&m)[V], int comp) {
+        const float *q = row + comp * n;
+        const float before = q[x == 0 ? g.nx - 1 : -1], after = q[x + V == g.nx ? V - g.nx : V];
+        if constexpr (V == 4) {
+          const float4 t = *reinterpret_cast<const float4 *>(q);
+          p[0] = t.y, p[1] = t.z, p[2] = t.w;
+          m[1] = t.x, m[2] = t.y, m[3] = t.z;
+        }
+        p[V - 1] = after;
+        m[0] = before;
+      };
+      // twice the component: d u_c1 / d x_a1 - d u_c2 / d x_a2
+      auto component = [&](const float (&up)[V], const float (&um)[V], const float (&vp)[V],
+                           const float (&vm)[V]) {
 #pragma unroll
-    for (int a = 0; a < D; ++a)
-      if (((g.walls >> a) & 1) && (p[a] == 0 || p[a] == dims[a] - 1)) wgt *= 0.5;
-    const double wz = diff(1, 0) - diff(0, 1);
-    double wx = 0.0, wy = 0.0;
-    if (D == 3) {
-      wx = diff(2, 1) - diff(1, 2);
-      wy = diff(0, 2) - diff(2, 0);
+        for (int k = 0; k < V; ++k) {
+          float s1, e1, s2, e2, s, e;
+          two_diff(up[k], um[k], s1, e1);
+          two_diff(vp[k], vm[k], s2, e2);
+          two_diff(s1, s2, s, e);
+          e += e1 - e2;
+          const bool wall =
+              plane || ((g.walls & 1) && ((k == 0 && x == 0) || (k == V - 1 && x + V == g.nx)));
+          if (wall) continue;
+          // NaN and infinities too
+          if (!(fabsf(s) >= 0x1p-45f && fabsf(s) <= 0x1p50f)) {
+            if (s != 0.f || e != 0.f) add_wide(&rare, up[k], um[k], vp[k], vm[k]);
+            continue;
+          }
+          const float q = s * s;
+          part.add(q, fmaf(e, e, fmaf(2.0f * s, e, fmaf(s, s, -q))));
+        }
+      };
+      float up[V], um[V], vp[V], vm[V];
+      load_x(up, um, 1);
+      load(vp, 0, yp);
+      load(vm, 0, ym);
+      component(up, um, vp, vm);
+      if (D == 3) {
+        load(up, 2, yp);
+        load(um, 2, ym);
+        load(vp, 1, zp);
+        load(vm, 1, zm);
+        component(up, um, vp, vm);
+        load(up, 0, zp);
+        load(um, 0, zm);
+        load_x(vp, vm, 2);
+        component(up, um, vp, vm);
+      }
+      if (g.walls) {
+        for (int k = 0; k < V; ++k)
+          if (plane || ((g.walls & 1) && (x + k == 0 || x + k == g.nx - 1)))
+            add_wall_node<D>(&rare, u, g, x + k, y, z);
+      }
     }
-    acc[0] += wgt * 0.5 * (wx * wx + wy * wy + wz * wz);
+    acc[0] += 0.125 * ((double)part.s + (double)part.e);
   }
+  acc[0] += rare;
   block_sum<1>(acc, partials + blockIdx.x);
 }
 
@@ -422,10 +558,16 @@ cudaError_t launch_diagnostics_blocks(int q, int storage, const void *f, const G
 cudaError_t launch_enstrophy(int d, const float *u, const Grid &g, int max_blocks,
                              double *partials, double *out, cudaStream_t st) {
   const int nb = red_blocks(g.n, max_blocks);
-  if (d == 2)
-    enstrophy_partial_kernel<2><<<nb, kRedThreads, 0, st>>>(u, g, partials);
+  // float4 rows: u starts nx ny nz floats into its allocation
+  const bool quads = g.nx % 4 == 0 && reinterpret_cast<uintptr_t>(u) % 16 == 0;
+  if (d == 2 && quads)
+    enstrophy_partial_kernel<2, 4><<<nb, kRedThreads, 0, st>>>(u, g, partials);
+  else if (d == 2)
+    enstrophy_partial_kernel<2, 1><<<nb, kRedThreads, 0, st>>>(u, g, partials);
+  else if (quads)
+    enstrophy_partial_kernel<3, 4><<<nb, kRedThreads, 0, st>>>(u, g, partials);
   else
-    enstrophy_partial_kernel<3><<<nb, kRedThreads, 0, st>>>(u, g, partials);
+    enstrophy_partial_kernel<3, 1><<<nb, kRedThreads, 0, st>>>(u, g, partials);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   finalize_kernel<<<1, kRedThreads, 0, st>>>(partials, nb, 1, out);
