@@ -849,14 +849,14 @@ int lb_mlp_train_step(lb_mlp *m, const void *X, const float *T, long long M, flo
   return mlp_backward(m, X, T, M, nullptr, 1, lr, loss);
 }
 
-// Closure scratch: the moment field (features of lb_closure_features and the
-// network of grids that are not whole row tiles), the predictions, and for
-// row-tile grids the feature source of the TMA-fed network with its map.
+// Closure scratch: the moment field (lb_closure_features), and for the step
+// (for_step) the feature source of the TMA-fed network with its map, or, on
+// the grids that it does not take, the moment field and the predictions.
 static int ensure_mom(lb_ctx *c, bool for_step) {
   const bool conv = for_step && lbrr::mlp_conv_supported(c->g);
   cudaError_t e = cudaSuccess;
   if (!conv && !c->mom) e = cudaMalloc(&c->mom, sizeof(float) * 10 * (size_t)c->g.n);
-  if (e == cudaSuccess && !conv && !c->ystd)  // the fused network writes no predictions
+  if (e == cudaSuccess && for_step && !conv && !c->ystd)
     e = cudaMalloc(&c->ystd, sizeof(float) * 17 * (size_t)c->g.n);
   if (e == cudaSuccess && conv && !c->xs) {
     e = cudaMalloc(&c->xs, lbrr::feature_source_bytes(c->g));
@@ -1004,7 +1004,7 @@ int lb_closure_step_trace(lb_ctx *c, float *trace, void *xs_out) {
   if (!trace || !xs_out) return fail(c, LB_EINVAL, "null trace or feature-source buffer");
   LB_NEED_DEVICE(c, trace);
   LB_NEED_DEVICE(c, xs_out);
-  if (!c->closure || !c->xs)
+  if (!c->closure || !c->xs || !lbrr::mlp_conv_rows(c->g))
     return fail(c, LB_EINVAL,
                 "needs a learned closure on a grid of whole 128-cell row tiles (lb_set_closure)");
   DeviceGuard dg(c->device);

@@ -193,12 +193,14 @@ cudaError_t launch_step_targets(const MlpDevice &p, const float *fpre, int ppre,
 cudaError_t launch_mlp_tc(const MlpDevice &p, const void *X, const float *mom, const Grid *g,
                           long long M, float *Y, int *status, int nblocks, cudaStream_t st,
                           float *H = nullptr);
-// The TMA-fed, pipelined forward pass (lbrr_mlp_conv.cu) for grids whose
-// rows are whole 128-cell tiles: the feature source xs (standardised moments,
+// The TMA-fed, pipelined forward pass (lbrr_mlp_conv.cu), for grids whose
+// rows are whole 128-cell tiles (mlp_conv_rows) and for others with little
+// padding: the feature source xs (standardised moments,
 // BF16, one-cell periodic halo, in the two 8-channel halves that kernel
 // reads: feature_source_bytes(g) bytes), its tensor map, and the network on
 // it. launch_export_features writes the feature source channels-last,
 // [(nx + 2)(ny + 2)(nz + 2)][16] BF16 (channels 10..15 zero).
+bool mlp_conv_rows(const Grid &g);
 bool mlp_conv_supported(const Grid &g);
 size_t feature_source_bytes(const Grid &g);
 cudaError_t make_feature_map(void *xs, const Grid &g, CUtensorMap *map);

@@ -1,13 +1,13 @@
-// Closure-network forward pass fused with the closure update, for grids whose
-// rows are whole 128-cell tiles, fed by the tensor memory accelerator (TMA)
-// and pipelined across tiles.
+// Closure-network forward pass fused with the closure update, fed by the tensor
+// memory accelerator (TMA) and pipelined across tiles of 128 cells: for rows of
+// whole tiles, and for other grids (FLAT) with tiles that run on across rows.
 //
 // Layer 1 of the network is a 3x3x3 convolution of the standardised moment
 // field: its 270 inputs for a cell are the 10 moments of the 27 cells around
 // it. A feature-source tensor holds those moments once per position of the
 // grid with a one-cell periodic halo (X = x + 1, Y = y + 1, Z = z + 1), BF16,
 // split in two halves of 8 channels, each half laid out [Z][Y][X][8] with
-// rows padded to nx + 8 positions:
+// rows padded to a multiple of 8 positions (nx + 8 for rows of whole tiles):
 //   half 0: moments 0..7 (rho - 1, ux, uy, uz, Pi xx, xy, xz, yy) at X;
 //   half 1: moments 8, 9 (Pi yz, zz) at X - 1, X and X + 1, then two ones
 //           (the constant input through which layer 1 adds its bias).
@@ -25,6 +25,15 @@
 // of all three dx. The weight operand of each MMA is W1's 16 matching
 // columns; at the centre row the two constant inputs meet b1 split into
 // BF16 b_hi + b_lo (b1 - b_hi - b_lo is below 2^-18 |b1|).
+//
+// FLAT: a tile is 128 consecutive positions of a plane, counted over its padded
+// rows, so that a neighbour row is again 136 consecutive positions, dy rows
+// further on; it is copied by one load per half of 17 chunks. The tile rows that
+// fall on the padding (8 of 72 positions at nx = 64) are computed and dropped,
+// and the rest of b1 meets the constant inputs of the row after the centre, so
+// that the bias is b1 to the bit. 64^3 takes 42 us a step; the moment
+// field, the network fed by threads (mlp_tc_kernel, one tile after another) and
+// the separate update, 119 (250^3: 1.42 and 6.91 ms).
 //
 // One persistent block per SM, nineteen warps:
 //   warp 0      TMA producer: per tile 2 tile loads (halves) for each of the 3 z
@@ -73,7 +82,10 @@ using namespace tc;
 constexpr int kCRows = 128;                         // cells per tile
 constexpr int kChunk = 8;                           // positions per 128-byte TMA row
 constexpr int kRowPos = 136;                        // staged positions x0 - 1 .. x0 + 134
-constexpr int kPadPos = 8;                          // padded row: nx + 8 positions
+// positions of a padded row: the halo, then a multiple of a chunk
+__host__ __device__ constexpr int row_pitch(int nx) {
+  return (nx + 2 + kChunk - 1) / kChunk * kChunk;
+}
 constexpr uint32_t kRowBytes = kRowPos * 16;        // one neighbour row of one half
 constexpr uint32_t kHalfBytes = 9 * kRowBytes;      // the 9 neighbour rows of one half
 constexpr uint32_t kStageBytes = 2 * kHalfBytes;
@@ -84,7 +96,7 @@ constexpr uint32_t kTxPart = 2 * kPartRows * kRowBytes;  // bytes a part receive
 constexpr int kMmas1 = 18;                          // layer-1 MMAs, K = 16 each
 constexpr uint32_t kW1Bytes = 2 * kMlpHidden * 16;  // W1 block of one layer-1 MMA
 static_assert(kRowPos % kChunk == 0 && kRowPos >= kCRows + 2, "staged row covers the taps");
-static_assert(kPadPos % kChunk == 0 && kPadPos >= kRowPos - kCRows, "last box inside the row");
+static_assert(row_pitch(kCRows) == kRowPos, "last box inside the row");
 constexpr uint32_t kPopBytes = 27 * kCRows * 4;    // populations of one tile, [27][128]
 constexpr int kGroups = 4;                          // epilogue groups
 constexpr int kIssuers = 2;                         // layer-1 MMA warps
@@ -127,7 +139,15 @@ __device__ __forceinline__ void mbar_expect_tx(uint32_t mbar, uint32_t bytes) {
   asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(mbar), "r"(bytes)
                : "memory");
 }
-// 5-D tiled TMA load (coordinates innermost first), completing on mbar
+// 3-D and 5-D tiled TMA loads (coordinates innermost first), completing on mbar
+__device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap *map, int c0, int c1,
+                                            int c2, uint32_t mbar) {
+  asm volatile(
+      "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
+      " [%0], [%1, {%2, %3, %4}], [%5];\n" ::"r"(dst),
+      "l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(c1), "r"(c2), "r"(mbar)
+      : "memory");
+}
 __device__ __forceinline__ void tma_load_5d(uint32_t dst, const CUtensorMap *map, int c0, int c1,
                                             int c2, int c3, int c4, uint32_t mbar) {
   asm volatile(
@@ -198,7 +218,7 @@ __device__ __forceinline__ void load_acc32(uint32_t taddr, uint32_t (&v)[32]) {
 // TRACE: also trace[cell][0..63], [64..127] (the FP32 activations of layers
 // 1 and 2 before their BF16 rounding) and [128..144] (the 17 standardised
 // predictions) of every cell.
-template <int PARITY, typename IDX, bool TRACE = false>
+template <int PARITY, typename IDX, bool TRACE = false, bool FLAT = false>
 __global__ void __launch_bounds__(kConvThreads, 1)
     mlp_conv_kernel(MlpDevice p, const __grid_constant__ CUtensorMap xs_map, const Grid g,
                     float *__restrict__ f, const float om1, unsigned long long *fallbacks,
@@ -239,6 +259,11 @@ __global__ void __launch_bounds__(kConvThreads, 1)
       w[6] = __bfloat16_as_ushort(hi);
       w[7] = __bfloat16_as_ushort(__float2bfloat16_rn(p.b1[n] - __bfloat162float(hi)));
     }
+    if (FLAT && kind == 1 && h == 1 && r9 == 5) {  // what b_hi + b_lo leave of b1
+      const float lo = p.b1[n] - __bfloat162float(__float2bfloat16_rn(p.b1[n]));
+      w[6] = __bfloat16_as_ushort(
+          __float2bfloat16_rn(lo - __bfloat162float(__float2bfloat16_rn(lo))));
+    }
     *reinterpret_cast<uint4 *>(smem + kSmW1 + mq * kW1Bytes + h * 1024 + n * 16) =
         make_uint4(w[0] | ((uint32_t)w[1] << 16), w[2] | ((uint32_t)w[3] << 16),
                    w[4] | ((uint32_t)w[5] << 16), w[6] | ((uint32_t)w[7] << 16));
@@ -278,7 +303,11 @@ __global__ void __launch_bounds__(kConvThreads, 1)
   fence_after();
   const uint32_t tmem = *tmem_slot;
   const uint32_t lim = wait_limit(status);
-  const long long ntiles = g.n / kCRows;
+  // tiles of a row, or of a plane
+  const uint32_t pitch = (uint32_t)row_pitch(g.nx);
+  const uint32_t tpr =
+      FLAT ? (pitch * (uint32_t)g.ny + kCRows - 1) / kCRows : (uint32_t)g.nx / kCRows;
+  const long long ntiles = FLAT ? (long long)tpr * g.nz : g.n / kCRows;
   const uint32_t sw1 = smem_u32(smem + kSmW1), sw2 = smem_u32(smem + kSmW2);
   const uint32_t sw3 = smem_u32(smem + kSmW3), sa1 = smem_u32(smem + kOffA1);
 
@@ -293,10 +322,10 @@ __global__ void __launch_bounds__(kConvThreads, 1)
         const int j = issued / kParts, s = j % kStages, use = j / kStages;
         // tile -> (x0, y, z) in 32-bit arithmetic (the launcher keeps the
         // tile count below 2^31)
-        const uint32_t t = (uint32_t)tile, tpr = (uint32_t)g.nx / kCRows;
-        const uint32_t row = t / tpr;
-        const int x0 = (int)(t - row * tpr) * kCRows;
-        const int y = (int)(row % (uint32_t)g.ny), z = (int)(row / (uint32_t)g.ny);
+        const uint32_t t = (uint32_t)tile, row = t / tpr;
+        const int x0 = (int)(t - row * tpr) * kCRows;  // FLAT: the position in plane z = row
+        const int y = FLAT ? 0 : (int)(row % (uint32_t)g.ny);
+        const int z = (int)(FLAT ? row : row / (uint32_t)g.ny);
         // part k: the z plane Z = z + k (padded), rows Y = y .. y + 2, chunks from X = x0
         for (int k = 0; k < kParts; ++k) {
           const int b = s * kParts + k;
@@ -307,9 +336,19 @@ __global__ void __launch_bounds__(kConvThreads, 1)
           }
           mbar_expect_tx(bar(kBarFull + b), kTxPart);
 #pragma unroll
-          for (int h = 0; h < 2; ++h)
-            tma_load_5d(sa1 + s * kStageBytes + h * kHalfBytes + k * kPartRows * kRowBytes,
-                        &xs_map, 0, x0 / kChunk, y, z + k * (3 / kParts), h, bar(kBarFull + b));
+          for (int h = 0; h < 2; ++h) {
+            const uint32_t dst = sa1 + s * kStageBytes + h * kHalfBytes + k * kPartRows * kRowBytes;
+            if constexpr (FLAT) {  // neighbour rows Y = y .. y + 2 of the plane
+              const int c0 = (z + k) * (g.ny + 2) * (int)(pitch / kChunk) + x0 / kChunk;
+#pragma unroll
+              for (int dy = 0; dy < kPartRows; ++dy)
+                tma_load_3d(dst + dy * kRowBytes, &xs_map, 0, c0 + dy * (int)(pitch / kChunk), h,
+                            bar(kBarFull + b));
+            } else {
+              tma_load_5d(dst, &xs_map, 0, x0 / kChunk, y, z + k * (3 / kParts), h,
+                          bar(kBarFull + b));
+            }
+          }
           ++issued;
         }
       }
@@ -374,7 +413,6 @@ __global__ void __launch_bounds__(kConvThreads, 1)
     // columns: c1 the layer-1 accumulator, then the BF16 rows h1 and h2 (A
     // operands of layers 2 and 3) in its first 32 columns; c2 layer 2, then 3
     const uint32_t c1 = 128 * eg, c2 = 128 * eg + 64, c3 = c2;
-    const uint32_t tpr = (uint32_t)g.nx / kCRows;
     uint32_t ph2 = 0, ph3 = 0;
     int j = eg;  // the block's tile index
     for (long long tile = blockIdx.x + (long long)eg * gridDim.x; tile < ntiles;
@@ -382,11 +420,22 @@ __global__ void __launch_bounds__(kConvThreads, 1)
       // this row's cell; its 27 populations go to shared memory while the
       // network runs (each cell reads only locations no other cell touches)
       const uint32_t t = (uint32_t)tile, row = t / tpr;
-      const int x = (int)(t - row * tpr) * kCRows + r;
-      const int y = (int)(row % (uint32_t)g.ny), z = (int)(row / (uint32_t)g.ny);
+      int x = (int)(t - row * tpr) * kCRows + r, y, z;
+      if (FLAT) {
+        z = (int)row;
+        y = (int)((uint32_t)x / pitch);
+        x -= y * (int)pitch;
+      } else {
+        y = (int)(row % (uint32_t)g.ny);
+        z = (int)(row / (uint32_t)g.ny);
+      }
+      const bool cell = !FLAT || (x < g.nx && y < g.ny);  // not on the padding
+      if (cell) {
 #pragma unroll
-      for (int i = 0; i < 27; ++i)
-        cp_async4(spop + i * kCRows * 4, f + closure_read_offset<PARITY, IDX>(g, x, y, z, i));
+        for (int i = 0; i < 27; ++i)
+          cp_async4(spop + i * kCRows * 4, f + closure_read_offset<PARITY, IDX>(g, x, y, z, i));
+      }
+      if (FLAT) __syncwarp();
       cp_async_commit();
       bool ok = mbar_wait(bar(kBarAcc1F + eg), (j / kGroups) & 1, lim);
       if (group_any(eg, !ok || *abort_flag)) {
@@ -459,11 +508,14 @@ __global__ void __launch_bounds__(kConvThreads, 1)
 #pragma unroll
         for (int k = 0; k < kMlpOutUsed; ++k) trace_row[2 * kMlpHidden + k] = yk[k];
       cp_async_wait_all();
-      float df[27];
+      if (cell) {
+        float df[27];
 #pragma unroll
-      for (int i = 0; i < 27; ++i) df[i] = pop[i * kCRows];
-      closure_update_cell_df<PARITY, IDX>(sb + 2 * kMlpHidden + kMlpOut, f, g, om1, x, y, z, df,
-                                          yk, fallbacks, bound, dead_zone);
+        for (int i = 0; i < 27; ++i) df[i] = pop[i * kCRows];
+        closure_update_cell_df<PARITY, IDX>(sb + 2 * kMlpHidden + kMlpOut, f, g, om1, x, y, z, df,
+                                            yk, fallbacks, bound, dead_zone);
+      }
+      if (FLAT) __syncwarp();
     }
     cp_async_wait_all();  // no copy into shared memory outlives the block
   }
@@ -537,9 +589,9 @@ __global__ void __launch_bounds__(kFsThreads)
   s89[threadIdx.x] = w[4];
   __syncthreads();
   if (valid && threadIdx.x >= 1 && threadIdx.x <= kFsOut) {
-    const long long o = row * (g.nx + kPadPos) + X;
+    const long long o = row * row_pitch(g.nx) + X;
     xs[o] = make_uint4(w[0], w[1], w[2], w[3]);
-    xs[(long long)pz * py * (g.nx + kPadPos) + o] =
+    xs[(long long)pz * py * row_pitch(g.nx) + o] =
         make_uint4(s89[threadIdx.x - 1], w[4], s89[threadIdx.x + 1], 0x3F803F80u);  // 1.0, 1.0
   }
 }
@@ -551,17 +603,27 @@ __global__ void __launch_bounds__(256)
   const long long px = g.nx + 2, py = g.ny + 2, pz = g.nz + 2;
   const long long q = (long long)blockIdx.x * 256 + threadIdx.x;
   if (q >= px * py * pz) return;
-  const long long o = (q / px) * (g.nx + kPadPos) + q % px;
+  const long long o = (q / px) * row_pitch(g.nx) + q % px;
   out[2 * q] = xs[o];
-  out[2 * q + 1] = make_uint4(xs[pz * py * (g.nx + kPadPos) + o].y, 0u, 0u, 0u);
+  out[2 * q + 1] = make_uint4(xs[pz * py * row_pitch(g.nx) + o].y, 0u, 0u, 0u);
 }
 
 }  // namespace
 
-bool mlp_conv_supported(const Grid &g) { return g.nx % kCRows == 0 && g.walls == 0; }
+bool mlp_conv_rows(const Grid &g) { return g.nx % kCRows == 0 && g.walls == 0; }
+
+// Rows of whole tiles, and other grids whose padding is small enough for the
+// feature source to take no more memory than the predictions (17 floats a
+// cell) of the separate network, as it is where no extent is below 14. Times of
+// a step, this and the separate network: 14^3 18.5 and 22.0 us, 24 x 12 x 12
+// 18.5 and 20.9, 30^3 18.6 and 30.4, 96^3 106 and 406, 160 x 100 x 90 155 and
+// 660.
+bool mlp_conv_supported(const Grid &g) {
+  return mlp_conv_rows(g) || (g.walls == 0 && feature_source_bytes(g) <= 68 * (size_t)g.n);
+}
 
 size_t feature_source_bytes(const Grid &g) {
-  return 2 * (size_t)(g.nx + kPadPos) * (size_t)(g.ny + 2) * (size_t)(g.nz + 2) * 16;
+  return 2 * (size_t)row_pitch(g.nx) * (size_t)(g.ny + 2) * (size_t)(g.nz + 2) * 16;
 }
 
 cudaError_t make_feature_map(void *xs, const Grid &g, CUtensorMap *map) {
@@ -574,13 +636,25 @@ cudaError_t make_feature_map(void *xs, const Grid &g, CUtensorMap *map) {
     if (e != cudaSuccess || q != cudaDriverEntryPointSuccess || !fn) return cudaErrorNotSupported;
     encode = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(fn);
   }
+  const cuuint32_t estr[5] = {1, 1, 1, 1, 1};
+  if (!mlp_conv_rows(g)) {  // [half][chunk of all rows][8 positions x 8 channels]
+    const cuuint64_t chunks =
+        (cuuint64_t)(row_pitch(g.nx) / kChunk) * ((cuuint64_t)g.ny + 2) * ((cuuint64_t)g.nz + 2);
+    const cuuint64_t dims[3] = {8 * kChunk, chunks, 2};
+    const cuuint64_t strides[2] = {16 * kChunk, 16 * kChunk * chunks};
+    const cuuint32_t box[3] = {8 * kChunk, kRowPos / kChunk, 1};
+    const CUresult r = encode(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, xs, dims, strides, box,
+                              estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
+                              CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+                              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
+  }
   // [half][Z][Y][chunk][8 positions x 8 channels]
-  const cuuint64_t rowb = (cuuint64_t)(g.nx + kPadPos) * 16;
-  const cuuint64_t dims[5] = {8 * kChunk, (cuuint64_t)(g.nx + kPadPos) / kChunk,
+  const cuuint64_t rowb = (cuuint64_t)row_pitch(g.nx) * 16;
+  const cuuint64_t dims[5] = {8 * kChunk, (cuuint64_t)row_pitch(g.nx) / kChunk,
                               (cuuint64_t)g.ny + 2, (cuuint64_t)g.nz + 2, 2};
   const cuuint64_t strides[4] = {16 * kChunk, rowb, rowb * dims[2], rowb * dims[2] * dims[3]};
   const cuuint32_t box[5] = {8 * kChunk, kRowPos / kChunk, 3, 3 / kParts, 1};
-  const cuuint32_t estr[5] = {1, 1, 1, 1, 1};
   const CUresult r = encode(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, xs, dims, strides, box,
                             estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
                             CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
@@ -606,16 +680,24 @@ cudaError_t launch_mlp_conv_step(const MlpDevice &p, const CUtensorMap &map, con
                                  float *f, float om1, int parity, unsigned long long *fallbacks,
                                  float bound, float dead_zone, int *status, int nblocks,
                                  cudaStream_t st, float *trace) {
+  const bool flat = !mlp_conv_rows(g);
+  if (flat && trace) return cudaErrorInvalidValue;
   // 32-bit element offsets where every slot of the store is addressable so
-  auto kern = trace ? (parity ? mlp_conv_kernel<1, long long, true>
+  const bool narrow = 27 * g.n < (1LL << 31);
+  auto kern = flat ? (narrow ? (parity ? mlp_conv_kernel<1, int, false, true>
+                                       : mlp_conv_kernel<0, int, false, true>)
+                             : (parity ? mlp_conv_kernel<1, long long, false, true>
+                                       : mlp_conv_kernel<0, long long, false, true>))
+              : trace ? (parity ? mlp_conv_kernel<1, long long, true>
                               : mlp_conv_kernel<0, long long, true>)
-              : 27 * g.n < (1LL << 31) ? (parity ? mlp_conv_kernel<1, int> : mlp_conv_kernel<0, int>)
+              : narrow ? (parity ? mlp_conv_kernel<1, int> : mlp_conv_kernel<0, int>)
                                        : (parity ? mlp_conv_kernel<1, long long>
                                                  : mlp_conv_kernel<0, long long>);
   cudaError_t e =
       cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kConvSmem);
   if (e != cudaSuccess) return e;
-  const long long tiles = g.n / kCRows;
+  const long long tiles =
+      flat ? ((long long)row_pitch(g.nx) * g.ny + kCRows - 1) / kCRows * g.nz : g.n / kCRows;
   if (tiles >= (1LL << 31)) return cudaErrorInvalidValue;
   const int nb = (int)(tiles < nblocks ? tiles : nblocks);
   if (nb < 1) return cudaSuccess;

@@ -47,12 +47,7 @@ constexpr uint32_t kOffSA1 = kOffSW3 + kW3Bytes;
 constexpr uint32_t kOffSA2 = kOffSA1 + kA1Bytes;
 constexpr uint32_t kOffSA3 = kOffSA2 + kA2Bytes;
 constexpr uint32_t kOffMisc = kOffSA3 + kA2Bytes;  // mbarrier, TMEM address, biases
-// staged moment field of a row-segment tile: 9 neighbour rows x 10 moments,
-// x0 - 1 .. x0 + 128 at positions 3 .. 132 (interior 16-byte aligned at 4)
-constexpr int kMsLen = 136;
-constexpr uint32_t kOffMs = kOffMisc + 1024;
-constexpr uint32_t kMsBytes = 9 * kMlpMoments * kMsLen * 4;  // 48960
-constexpr uint32_t kTcSmem = kOffMs + kMsBytes;
+constexpr uint32_t kTcSmem = kOffMisc + 1024;
 
 __device__ __forceinline__ uint32_t pack2(float lo, float hi) { return pack_bf16(lo, hi); }
 
@@ -84,49 +79,7 @@ __device__ __forceinline__ void hidden_epilogue(uint32_t taddr, const float *bia
   }
 }
 
-// Standardised feature f = 10 nb + k of row r from the staged moment rows
-// ms[row9 * 10 + k] (row9 = (dy+1) + 3 (dz+1)) at x offset 4 + r + dx.
-template <int F>
-__device__ __forceinline__ float staged_feature(const MlpDevice &p, const float *ms, int r) {
-  constexpr int nb = F / kMlpMoments, k = F % kMlpMoments;
-  constexpr int dx = nb % 3 - 1, row9 = nb / 3;
-  return (ms[(row9 * kMlpMoments + k) * kMsLen + 4 + r + dx] - p.in_mean[k]) * p.in_inv_std[k];
-}
-
-template <int F>
-__device__ __forceinline__ uint32_t staged_pair(const MlpDevice &p, const float *ms, int r) {
-  if constexpr (F >= kMlpInUsed)
-    return 0u;
-  else
-    return pack2(staged_feature<F>(p, ms, r), staged_feature<F + 1>(p, ms, r));
-}
-
-// Chunks KB0 .. KB0 + 17 (8 features each) of row r, as 16-byte stores.
-template <int KB0, int KB = KB0>
-__device__ __forceinline__ void staged_chunks(const MlpDevice &p, const float *ms,
-                                              unsigned char *a1, int r) {
-  if constexpr (KB < KB0 + kMlpIn / 16) {
-    uint4 q;
-    q.x = staged_pair<8 * KB>(p, ms, r);
-    q.y = staged_pair<8 * KB + 2>(p, ms, r);
-    q.z = staged_pair<8 * KB + 4>(p, ms, r);
-    q.w = staged_pair<8 * KB + 6>(p, ms, r);
-    *reinterpret_cast<uint4 *>(a1 + cm_offset(r, 8 * KB, kMlpIn)) = q;
-    staged_chunks<KB0, KB + 1>(p, ms, a1, r);
-  }
-}
-
-// Features of row r into the A1 tile: half 0 writes chunks 0..17, half 1
-// chunks 18..35 (the last ones hold the zero padding).
-__device__ __forceinline__ void features_staged(const MlpDevice &p, const float *ms,
-                                                unsigned char *a1, int r, int half) {
-  if (half == 0)
-    staged_chunks<0>(p, ms, a1, r);
-  else
-    staged_chunks<kMlpIn / 16>(p, ms, a1, r);
-}
-
-// Same from the moment field in global memory (any grid shape).
+// Standardised features of row r from the moment field in global memory.
 __device__ __forceinline__ void features_gather(const MlpDevice &p, const float *mom,
                                                 const Grid &g, long long cell,
                                                 unsigned char *a1, int r, int half) {
@@ -153,8 +106,7 @@ __device__ __forceinline__ void features_gather(const MlpDevice &p, const float 
 
 // FROM_MOM: rows are the cells of a grid and their features are built from
 // the moment field mom [10][N]; outputs y[k][cell] for the 17 used outputs.
-// When nx is a multiple of 128 a tile is one row segment and the 9 x 10
-// moment rows around it are first staged in shared memory with 16-byte loads.
+// (Small grids only: lbrr_mlp_conv.cu takes the others.)
 // Otherwise rows are X [M][288] (BF16) and outputs Y [M][32].
 // TRACE (rows X only): also H[row][0..63] and H[row][64..127], the FP32
 // activations of layers 1 and 2 before their BF16 rounding.
@@ -169,7 +121,6 @@ __global__ void __launch_bounds__(kTcThreads, 1)
   uint64_t *mbar = reinterpret_cast<uint64_t *>(smem + kOffMisc);
   uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(smem + kOffMisc + 8);
   float *sb = reinterpret_cast<float *>(smem + kOffMisc + 64);  // b1, b2, b3 (160)
-  float *ms = reinterpret_cast<float *>(smem + kOffMs);
   const uint32_t mbar_a = smem_u32(mbar);
 
   // ---- weights into the canonical layout; biases
@@ -216,53 +167,13 @@ __global__ void __launch_bounds__(kTcThreads, 1)
   uint32_t phase = 0;
   bool ok = true;
   const long long ntiles = (M + kTcRows - 1) / kTcRows;
-  const long long n = g.n;
-  const bool staged = FROM_MOM && (g.nx % kTcRows == 0);
-
-  // asynchronous copy of the 9 x 10 moment rows around a row-segment tile
-  // (x0 - 1 .. x0 + 128, periodic) into ms
-  auto stage = [&](long long t) {
-    const long long first = t * kTcRows;
-    const int x0 = (int)(first % g.nx);
-    const long long yz = first / g.nx;
-    const int y = (int)(yz % g.ny), z = (int)(yz / g.ny);
-    for (int q = tid; q < 9 * kMlpMoments * (kTcRows / 4); q += kTcThreads) {
-      const int sgm = q / (kTcRows / 4), j = q - sgm * (kTcRows / 4);
-      const int row9 = sgm / kMlpMoments, k = sgm - row9 * kMlpMoments;
-      const int yy = wrap_add(y, row9 % 3 - 1, g.ny), zz = wrap_add(z, row9 / 3 - 1, g.nz);
-      const float *src = mom + k * n + ((long long)zz * g.ny + yy) * g.nx + x0 + 4 * j;
-      const unsigned d = smem_u32(ms + sgm * kMsLen + 4 + 4 * j);
-      asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(d), "l"(src) : "memory");
-    }
-    for (int q = tid; q < 9 * kMlpMoments * 2; q += kTcThreads) {
-      const int sgm = q >> 1, side = q & 1;
-      const int row9 = sgm / kMlpMoments, k = sgm - row9 * kMlpMoments;
-      const int yy = wrap_add(y, row9 % 3 - 1, g.ny), zz = wrap_add(z, row9 / 3 - 1, g.nz);
-      const int xx = side ? (x0 + kTcRows == g.nx ? 0 : x0 + kTcRows)
-                          : (x0 == 0 ? g.nx - 1 : x0 - 1);
-      const float *src = mom + k * n + ((long long)zz * g.ny + yy) * g.nx + xx;
-      const unsigned d = smem_u32(ms + sgm * kMsLen + (side ? 4 + kTcRows : 3));
-      asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(d), "l"(src) : "memory");
-    }
-  };
-  if (staged && (long long)blockIdx.x < ntiles) stage(blockIdx.x);
 
   for (long long tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x) {
     const long long row = tile * kTcRows + r;
     const bool valid = row < M;
     unsigned char *a1 = smem + kOffSA1;
     // ---- input rows
-    if (FROM_MOM && staged) {
-      // the moment rows of this tile were requested (cp.async) before the
-      // previous tile's products; wait for them, build the features, then
-      // request the next tile's rows so that they arrive during this tile's
-      // products and epilogues
-      asm volatile("cp.async.wait_all;\n" ::: "memory");
-      __syncthreads();
-      features_staged(p, ms, a1, r, half);
-      __syncthreads();
-      if (tile + gridDim.x < ntiles) stage(tile + gridDim.x);
-    } else if (FROM_MOM) {
+    if (FROM_MOM) {
       if (valid) {
         features_gather(p, mom, g, row, a1, r, half);
       } else {
@@ -347,11 +258,10 @@ __global__ void __launch_bounds__(kTcThreads, 1)
       }
     }
     fence_before();
-    __syncthreads();  // the next tile overwrites A1, the staged moments and the accumulators
+    __syncthreads();  // the next tile overwrites A1 and the accumulators
     fence_after();
   }
 
-  asm volatile("cp.async.wait_all;\n" ::: "memory");  // no copy outlives the block
   if (!ok) {
     if (tid == 0) atomicExch(status, 1);
     // let any MMA still in flight finish before the memory goes away
