@@ -40,31 +40,72 @@ __global__ void __launch_bounds__(kAux)
 }
 
 // -------------------------------------------------------------- features --
-__device__ __forceinline__ long long nb_cell(const Grid &g, int x, int y, int z, int nb) {
-  const int dx = nb % 3 - 1, dy = (nb / 3) % 3 - 1, dz = nb / 9 - 1;
-  return ((long long)wrap_add(z, dz, g.nz) * g.ny + wrap_add(y, dy, g.ny)) * g.nx +
-         wrap_add(x, dx, g.nx);
-}
+// Bound by its output: 576 B a cell against 40 B of moments. With a thread
+// writing its cell's row 4 bytes at a time the lines of 32 rows were open at
+// once and 64^3 took 315 us. So a block takes kFeatX cells of kFeatY rows of
+// a plane, forms the standardised moments of these and their neighbours once,
+// packed two to a word as the features hold them, and then kFeatChunks threads
+// to a cell each gather 4 words of their own fixed place in the feature row:
+// 16-byte stores, consecutive along the rows. 35 us.
+constexpr int kFeatX = 32, kFeatY = 4;                // cells of a block
+constexpr int kFeatChunks = kMlpIn / 8;               // 16-byte chunks of a feature row
+constexpr int kFeatThreads = 8 * kFeatChunks;         // 8 cells at a time
+constexpr int kFeatPairs = kMlpMoments / 2;           // words of a cell
+constexpr int kFeatRow = (kFeatX + 2) * kFeatPairs;   // words of a staged row
+static_assert(kFeatX % 8 == 0, "the cells taken at a time lie in one row");
 
-__global__ void __launch_bounds__(kAux)
-    features_kernel(MlpDevice p, const float *__restrict__ mom, const Grid g,
-                    __nv_bfloat16 *__restrict__ X) {
-  const long long cell = (long long)blockIdx.x * kAux + threadIdx.x;
-  if (cell >= g.n) return;
-  int x, y, z;
-  cell_coords(cell, g, x, y, z);
+__global__ void __launch_bounds__(kFeatThreads)
+    features_kernel(MlpDevice p, const float *__restrict__ mom, const Grid g, const int tiles_x,
+                    const int tiles_y, uint4 *__restrict__ X) {
+  __shared__ uint32_t words[3 * (kFeatY + 2) * kFeatRow];
   const long long n = g.n;
-  uint32_t *row = reinterpret_cast<uint32_t *>(X + cell * kMlpIn);
-  for (int nb = 0; nb < 27; ++nb) {
-    const long long c = nb_cell(g, x, y, z, nb);
+  const unsigned b = blockIdx.x, bx = b % (unsigned)tiles_x, byz = b / (unsigned)tiles_x;
+  const int x0 = (int)bx * kFeatX, y0 = (int)(byz % (unsigned)tiles_y) * kFeatY;
+  const int z = (int)(byz / (unsigned)tiles_y);
+  const int nx = min(kFeatX, g.nx - x0), ny = min(kFeatY, g.ny - y0);
+  for (int q = threadIdx.x; q < 3 * (kFeatY + 2) * (kFeatX + 2); q += kFeatThreads) {
+    const int row = q / (kFeatX + 2), px = q - row * (kFeatX + 2);
+    const int pz = row / (kFeatY + 2), py = row - pz * (kFeatY + 2);
+    if (px > nx + 1 || py > ny + 1) continue;
+    const int x = x0 + px - 1, y = y0 + py - 1;
+    const long long c = ((long long)wrap_add(z, pz - 1, g.nz) * g.ny +
+                         (y < 0 ? g.ny - 1 : y == g.ny ? 0 : y)) * g.nx +
+                        (x < 0 ? g.nx - 1 : x == g.nx ? 0 : x);
 #pragma unroll
     for (int k = 0; k < kMlpMoments; k += 2) {
       const float v0 = (__ldg(mom + k * n + c) - p.in_mean[k]) * p.in_inv_std[k];
       const float v1 = (__ldg(mom + (k + 1) * n + c) - p.in_mean[k + 1]) * p.in_inv_std[k + 1];
-      row[(kMlpMoments * nb + k) / 2] = pack_bf16(v0, v1);
+      words[row * kFeatRow + px * kFeatPairs + k / 2] = pack_bf16(v0, v1);
     }
   }
-  for (int k = kMlpInUsed; k < kMlpIn; k += 2) row[k / 2] = 0u;
+  __syncthreads();
+  const bool wide = reinterpret_cast<uintptr_t>(X) % 16 == 0;  // else 4-byte stores
+  const int chunk = threadIdx.x % kFeatChunks, first = threadIdx.x / kFeatChunks;
+  int place[4];  // of the chunk's words, from the staged row and position of the cell's (-1, -1, -1)
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const int w = 4 * chunk + k, nb = w / kFeatPairs;
+    place[k] = nb < 27 ? ((nb / 9) * (kFeatY + 2) + (nb / 3) % 3) * kFeatRow +
+                             (nb % 3) * kFeatPairs + w - nb * kFeatPairs
+                       : -1;  // zero padding
+  }
+  for (int q = first; q < kFeatX * kFeatY; q += kFeatThreads / kFeatChunks) {
+    const int x = q % kFeatX, y = q / kFeatX;
+    if (x >= nx || y >= ny) continue;
+    const uint32_t *w = words + y * kFeatRow + x * kFeatPairs;
+    uint4 v;
+    v.x = place[0] < 0 ? 0u : w[place[0]];
+    v.y = place[1] < 0 ? 0u : w[place[1]];
+    v.z = place[2] < 0 ? 0u : w[place[2]];
+    v.w = place[3] < 0 ? 0u : w[place[3]];
+    uint4 *dst = X + (((long long)z * g.ny + y0 + y) * g.nx + x0 + x) * kFeatChunks + chunk;
+    if (wide) {
+      *dst = v;
+    } else {
+      uint32_t *d = reinterpret_cast<uint32_t *>(dst);
+      d[0] = v.x, d[1] = v.y, d[2] = v.z, d[3] = v.w;
+    }
+  }
 }
 
 // --------------------------------------------------------------- targets --
@@ -97,21 +138,31 @@ __device__ __forceinline__ void hermite_analysis(const float (&d)[27], float (&A
       ana1(axy[a][b][0], axy[a][b][1], axy[a][b][2], A[a][b][0], A[a][b][1], A[a][b][2]);
 }
 
-// Row `cell` of a target matrix: the order 3..6 coefficients of A divided by
-// div * out_scale, zero padded.
+// The target rows of a warp's 32 cells first .. first + 31 (those below n), the
+// order 3..6 coefficients of A divided by div * out_scale, zero padded. They go
+// through shared memory, so that a store writes one row of 128 bytes: with each
+// thread storing its own row, step_targets_kernel took 74 us at 64^3; 43.
 __device__ __forceinline__ void write_targets(const MlpDevice &p, const float (&A)[3][3][3],
-                                              float div, float *__restrict__ row) {
+                                              float div, long long first, long long n,
+                                              float *__restrict__ T) {
+  __shared__ float rows[kAux / 32][32][kMlpOutUsed];  // odd row length: no bank conflicts
+  const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
 #pragma unroll
   for (int k = 0; k < kMlpOutUsed; ++k)
-    row[k] = A[hi_pow(k, 0)][hi_pow(k, 1)][hi_pow(k, 2)] / (div * p.out_scale[k]);
-  for (int k = kMlpOutUsed; k < kMlpOut; ++k) row[k] = 0.f;
+    rows[warp][lane][k] = A[hi_pow(k, 0)][hi_pow(k, 1)][hi_pow(k, 2)] / (div * p.out_scale[k]);
+  __syncwarp();
+  const int count = n - first < 32 ? (int)(n - first) : 32;
+  float *dst = T + first * kMlpOut + lane;
+#pragma unroll 8
+  for (int k = 0; k < count; ++k) dst[k * kMlpOut] = lane < kMlpOutUsed ? rows[warp][k][lane] : 0.f;
 }
 
 __global__ void __launch_bounds__(kAux)
     targets_kernel(MlpDevice p, const float *__restrict__ f, const Grid g, const int parity,
                    float *__restrict__ T) {
-  const long long cell = (long long)blockIdx.x * kAux + threadIdx.x;
-  if (cell >= g.n) return;
+  const long long first = (long long)blockIdx.x * kAux + (threadIdx.x & ~31u);  // of the warp
+  if (first >= g.n) return;
+  const long long cell = min(first + threadIdx.x % 32, g.n - 1);
   int x, y, z;
   cell_coords(cell, g, x, y, z);
   float df[27], rr[27];
@@ -122,7 +173,7 @@ __global__ void __launch_bounds__(kAux)
   for (int i = 0; i < 27; ++i) rr[i] = df[i] - rr[i];
   float A[3][3][3];
   hermite_analysis(rr, A);
-  write_targets(p, A, 1.0f, T + cell * kMlpOut);
+  write_targets(p, A, 1.0f, first, g.n, T);
 }
 
 // Step-matching targets of coarse cell x: P_i(x) = post_i(x + xi_i) (logical
@@ -134,8 +185,9 @@ __global__ void __launch_bounds__(kAux)
     step_targets_kernel(MlpDevice p, const float *__restrict__ fpre, const int ppre,
                         const float *__restrict__ fpost, const int ppost, const Grid g,
                         const float om1, float *__restrict__ T) {
-  const long long cell = (long long)blockIdx.x * kAux + threadIdx.x;
-  if (cell >= g.n) return;
+  const long long first = (long long)blockIdx.x * kAux + (threadIdx.x & ~31u);  // of the warp
+  if (first >= g.n) return;
+  const long long cell = min(first + threadIdx.x % 32, g.n - 1);
   int x, y, z;
   cell_coords(cell, g, x, y, z);
   float df[27], r[27];
@@ -157,7 +209,7 @@ __global__ void __launch_bounds__(kAux)
   }
   float A[3][3][3];
   hermite_analysis(r, A);
-  write_targets(p, A, om1, T + cell * kMlpOut);
+  write_targets(p, A, om1, first, g.n, T);
 }
 
 // -------------------------------------------------------------- coarsen --
@@ -227,8 +279,9 @@ cudaError_t launch_moment_field(int storage, const void *f, const Grid &g, int p
 
 cudaError_t launch_features(const MlpDevice &p, const float *mom, const Grid &g, void *X,
                             cudaStream_t st) {
-  features_kernel<<<(unsigned)((g.n + kAux - 1) / kAux), kAux, 0, st>>>(
-      p, mom, g, static_cast<__nv_bfloat16 *>(X));
+  const int tx = (g.nx + kFeatX - 1) / kFeatX, ty = (g.ny + kFeatY - 1) / kFeatY;
+  features_kernel<<<(unsigned)((long long)tx * ty * g.nz), kFeatThreads, 0, st>>>(
+      p, mom, g, tx, ty, static_cast<uint4 *>(X));
   return cudaGetLastError();
 }
 
