@@ -3,6 +3,7 @@
 #pragma once
 
 #include <cuda.h>
+#include <cudaTypedefs.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
@@ -184,6 +185,8 @@ cudaError_t launch_coarsen(int storage_f, const void *ff, const Grid &gf, int pa
 cudaError_t launch_step_targets(const MlpDevice &p, const float *fpre, int ppre,
                                 const float *fpost, int ppost, const Grid &g, float om1, float *T,
                                 cudaStream_t st);
+// cuTensorMapEncodeTiled, or null where the driver has none.
+PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder();
 // Network forward on the tcgen05 tensor cores (lbrr_mlp_tc.cu). With mom:
 // rows are the cells of grid *g, features from the moment field, outputs the
 // 17 standardised predictions Y [17][N]. Without: rows X [M][288] BF16, Y

@@ -626,16 +626,21 @@ size_t feature_source_bytes(const Grid &g) {
   return 2 * (size_t)row_pitch(g.nx) * (size_t)(g.ny + 2) * (size_t)(g.nz + 2) * 16;
 }
 
-cudaError_t make_feature_map(void *xs, const Grid &g, CUtensorMap *map) {
-  static PFN_cuTensorMapEncodeTiled_v12000 encode = nullptr;
-  if (!encode) {
+PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder() {
+  static const PFN_cuTensorMapEncodeTiled_v12000 encode = [] {
     cudaDriverEntryPointQueryResult q;
     void *fn = nullptr;
-    cudaError_t e =
+    const cudaError_t e =
         cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000, cudaEnableDefault, &q);
-    if (e != cudaSuccess || q != cudaDriverEntryPointSuccess || !fn) return cudaErrorNotSupported;
-    encode = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(fn);
-  }
+    if (e != cudaSuccess || q != cudaDriverEntryPointSuccess) fn = nullptr;
+    return reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(fn);
+  }();
+  return encode;
+}
+
+cudaError_t make_feature_map(void *xs, const Grid &g, CUtensorMap *map) {
+  PFN_cuTensorMapEncodeTiled_v12000 encode = tensor_map_encoder();
+  if (!encode) return cudaErrorNotSupported;
   const cuuint32_t estr[5] = {1, 1, 1, 1, 1};
   if (!mlp_conv_rows(g)) {  // [half][chunk of all rows][8 positions x 8 channels]
     const cuuint64_t chunks =

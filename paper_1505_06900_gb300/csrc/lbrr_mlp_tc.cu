@@ -3,20 +3,32 @@
 // tiles of 128 rows, BF16 operands in shared memory, FP32 accumulators in
 // tensor memory (TMEM).
 //
-// One block per SM (persistent). The BF16 weights are staged once into shared
-// memory in the canonical K-major layout without swizzle: 8 x 8 "core
-// matrices" of 128 contiguous bytes (8 rows of 16 bytes), adjacent core
-// matrices along K 128 bytes apart (leading byte offset) and adjacent 8-row
-// groups K/8 * 128 bytes apart (stride byte offset). Per tile the 128 threads
-// write the 128 input rows (thread r owns row r = TMEM lane r) in the same
-// layout; one thread issues the K/16 MMAs of a layer (M = 128, N = 64, 64, 32)
-// and commits them to an mbarrier; the threads then read their row of the
-// accumulator (tcgen05.ld 32x32b), add the bias, apply tanh, round to BF16 and
-// write the next layer's input rows. TMEM columns: layer 1 at 0, layer 2 at 64,
-// layer 3 at 128 (256 allocated).
+// One block per SM (persistent), in two groups of 256 threads that take
+// alternate tiles. The BF16 weights are staged once into shared memory in the
+// canonical K-major layout without swizzle: 8 x 8 "core matrices" of 128
+// contiguous bytes (8 rows of 16 bytes), adjacent core matrices along K 128
+// bytes apart (leading byte offset) and adjacent 8-row groups K/8 * 128 bytes
+// apart (stride byte offset). A tile's 128 input rows come by TMA in boxes of 64
+// columns in the layout with 128-byte swizzle, the last 32 with 64-byte swizzle;
+// one thread of the group issues the MMAs of a layer (M = 128, N = 64, 64, 32)
+// and commits them to the group's mbarrier; the threads, two to a row (TMEM
+// lane), then read the accumulator (tcgen05.ld 32x32b), add the bias, apply
+// tanh and write the BF16 row back into TMEM (tcgen05.st), the A operand of the
+// next layer.
 //
-// Every mbarrier wait is bounded: on expiry the block records a timeout in
-// *status, waits (bounded) for its MMAs to drain, frees its TMEM and returns.
+// Reading X (576 B a row) bounds it. One tile after another, loads, three
+// products and epilogues in turn, 262144 rows took 101 us; now the rows of a
+// group's next tile are requested as soon as layer 1 has read the present one's,
+// and the two groups' chains overlap: 39 us (62 with the rows copied by the
+// threads, 16 bytes each, whose issue alone held a tile up for 4400 to 9000
+// cycles). Outputs go through shared memory, a row of 128 bytes to a store.
+//
+// Every mbarrier wait is bounded: on expiry the group records a timeout in
+// *status and waits (bounded) for its MMAs to drain before the block frees its
+// TMEM and returns.
+#include <cuda.h>
+#include <cudaTypedefs.h>
+
 #include <cstdint>
 
 #include "lbrr_launch.h"
@@ -31,34 +43,76 @@ namespace {
 using namespace tc;
 
 constexpr int kTcRows = 128;
-constexpr int kTcThreads = 256;  // two threads per row; warps w and w + 4 share TMEM lanes
-constexpr uint32_t kTmemCols = 256;
+constexpr int kGroupThreads = 256;  // two threads per row; warps w and w + 4 share TMEM lanes
+constexpr int kTcGroups = 2;
+constexpr int kTcThreads = kTcGroups * kGroupThreads;
+// TMEM columns of a group: layer 1 then 3, layer 2, the BF16 rows between them
+constexpr uint32_t kColGroup = 192, kCol1 = 0, kCol2 = 64, kColH = 128;
+constexpr uint32_t kTmemCols = 512;
 
-// shared-memory plan (bytes, all 1024-aligned)
+// shared-memory plan (bytes, all 1024-aligned up to the output rows)
 constexpr uint32_t kW1Bytes = kMlpHidden * kMlpIn * 2;        // 36864
 constexpr uint32_t kW2Bytes = kMlpHidden * kMlpHidden * 2;    // 8192
 constexpr uint32_t kW3Bytes = kMlpOut * kMlpHidden * 2;       // 4096
 constexpr uint32_t kA1Bytes = kTcRows * kMlpIn * 2;           // 73728
-constexpr uint32_t kA2Bytes = kTcRows * kMlpHidden * 2;       // 16384
+constexpr int kYRow = kMlpOut + 1;                            // odd: no bank conflicts
+constexpr uint32_t kYBytes = kTcRows * kYRow * 4;             // 16896
 constexpr uint32_t kOffSW1 = 0;
 constexpr uint32_t kOffSW2 = kOffSW1 + kW1Bytes;
 constexpr uint32_t kOffSW3 = kOffSW2 + kW2Bytes;
 constexpr uint32_t kOffSA1 = kOffSW3 + kW3Bytes;
-constexpr uint32_t kOffSA2 = kOffSA1 + kA1Bytes;
-constexpr uint32_t kOffSA3 = kOffSA2 + kA2Bytes;
-constexpr uint32_t kOffMisc = kOffSA3 + kA2Bytes;  // mbarrier, TMEM address, biases
+constexpr uint32_t kOffY = kOffSA1 + kTcGroups * kA1Bytes;
+constexpr uint32_t kOffMisc = kOffY + kTcGroups * kYBytes;  // mbarriers, TMEM address, biases
 constexpr uint32_t kTcSmem = kOffMisc + 1024;
+// the boxes of a tile in A1
+constexpr int kBoxCols = 64, kBoxes = kMlpIn / kBoxCols, kLastCols = kMlpIn - kBoxes * kBoxCols;
+constexpr uint32_t kBoxBytes = kTcRows * kBoxCols * 2;
+static_assert(kLastCols == 32, "64-byte rows");
+static_assert(kOffSA1 % 1024 == 0 && kA1Bytes % 1024 == 0, "swizzle atoms");
+
+// Descriptor of a K-major operand with swizzled rows of 128 or 64 bytes (8 rows
+// an atom, atoms contiguous); a K step of 16 columns moves its start address.
+__device__ __forceinline__ uint64_t sdesc_swizzled(uint32_t saddr, bool wide) {
+  return sdesc(saddr, 16, wide ? 1024 : 512) | ((uint64_t)(wide ? 2 : 4) << 61);
+}
+// 2-D tiled TMA load, completing on mbar
+__device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap *map, int c0, int c1,
+                                            uint32_t mbar) {
+  asm volatile(
+      "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
+      " [%0], [%1, {%2, %3}], [%4];\n" ::"r"(dst),
+      "l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(c1), "r"(mbar)
+      : "memory");
+}
+static_assert(kTcSmem <= 232448, "fits the shared memory of one block");
+
+__device__ __forceinline__ void group_sync(int g) {
+  asm volatile("bar.sync %0, %1;\n" ::"r"(1 + g), "n"(kGroupThreads) : "memory");
+}
+// the same, returning whether any thread of the group passed pred = true
+__device__ __forceinline__ bool group_any(int g, bool pred) {
+  uint32_t r;
+  asm volatile(
+      "{\n.reg .pred p, q;\nsetp.ne.u32 p, %1, 0;\nbar.red.or.pred q, %2, %3, p;\n"
+      "selp.u32 %0, 1, 0, q;\n}\n"
+      : "=r"(r)
+      : "r"((uint32_t)pred), "r"(1 + g), "n"(kGroupThreads)
+      : "memory");
+  return r != 0;
+}
 
 __device__ __forceinline__ uint32_t pack2(float lo, float hi) { return pack_bf16(lo, hi); }
 
-// Layer epilogue: tanh(acc + bias) of 32 of the 64 columns (half 0 or 1) into
-// row r of a K = 64 operand; with TRACE also the FP32 values into hrow[64].
+// Layer epilogue: tanh(acc + bias) of columns 32 half .. 32 half + 31, as BF16
+// into the 16 TMEM columns at dst; with TRACE also the FP32 values into
+// hrow[64].
 template <bool TRACE = false>
-__device__ __forceinline__ void hidden_epilogue(uint32_t taddr, const float *bias,
-                                                unsigned char *dst, int r, int half,
-                                                float *hrow = nullptr) {
+__device__ __forceinline__ void hidden_epilogue(uint32_t taddr, const float *bias, uint32_t dst,
+                                                int half, float *hrow = nullptr) {
+  uint32_t q[16];
 #pragma unroll
-  for (int c0 = 32 * half; c0 < 32 * half + 32; c0 += 16) {
+  for (int i = 0; i < 2; ++i) {
+    const int c0 = 32 * half + 16 * i;
     float v[16];
     tmem_ld16(taddr + c0, v);
 #pragma unroll
@@ -68,15 +122,10 @@ __device__ __forceinline__ void hidden_epilogue(uint32_t taddr, const float *bia
       for (int k = 0; k < 16; k += 4)
         *reinterpret_cast<float4 *>(hrow + c0 + k) = make_float4(v[k], v[k + 1], v[k + 2], v[k + 3]);
 #pragma unroll
-    for (int k = 0; k < 16; k += 8) {
-      uint4 q;
-      q.x = pack2(v[k], v[k + 1]);
-      q.y = pack2(v[k + 2], v[k + 3]);
-      q.z = pack2(v[k + 4], v[k + 5]);
-      q.w = pack2(v[k + 6], v[k + 7]);
-      *reinterpret_cast<uint4 *>(dst + cm_offset(r, c0 + k, kMlpHidden)) = q;
-    }
+    for (int k = 0; k < 16; k += 2) q[8 * i + k / 2] = pack2(v[k], v[k + 1]);
   }
+  tmem_st16(dst, q);
+  tmem_wait_st();
 }
 
 // Standardised features of row r from the moment field in global memory.
@@ -112,16 +161,46 @@ __device__ __forceinline__ void features_gather(const MlpDevice &p, const float 
 // activations of layers 1 and 2 before their BF16 rounding.
 template <bool FROM_MOM, bool TRACE = false>
 __global__ void __launch_bounds__(kTcThreads, 1)
-    mlp_tc_kernel(MlpDevice p, const __nv_bfloat16 *__restrict__ X,
-                  const float *__restrict__ mom, const Grid g, long long M,
+    mlp_tc_kernel(MlpDevice p, const __grid_constant__ CUtensorMap x_map,
+                  const __grid_constant__ CUtensorMap x_last, const float *__restrict__ mom, const Grid g, long long M,
                   float *__restrict__ Y, int *status, float *__restrict__ H) {
   extern __shared__ __align__(1024) unsigned char smem[];
   const int tid = threadIdx.x, warp = tid >> 5;
-  const int r = tid & (kTcRows - 1), half = tid >> 7;  // row, and which half of its work
+  const int gr = tid / kGroupThreads, gt = tid % kGroupThreads;
+  const int r = gt & (kTcRows - 1), half = gt >> 7;  // row, and which half of its work
+  // of each group: MMAs done, rows landed
   uint64_t *mbar = reinterpret_cast<uint64_t *>(smem + kOffMisc);
-  uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(smem + kOffMisc + 8);
+  uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(smem + kOffMisc + 16 * kTcGroups);
   float *sb = reinterpret_cast<float *>(smem + kOffMisc + 64);  // b1, b2, b3 (160)
-  const uint32_t mbar_a = smem_u32(mbar);
+  unsigned char *a1 = smem + kOffSA1 + gr * kA1Bytes;
+  float *ys = reinterpret_cast<float *>(smem + kOffY + gr * kYBytes);
+  const uint32_t mbar_a = smem_u32(mbar + gr), mbar_x = smem_u32(mbar + kTcGroups + gr);
+  const long long ntiles = (M + kTcRows - 1) / kTcRows;
+  const long long stride = (long long)kTcGroups * gridDim.x;
+
+  long long tile = blockIdx.x + (long long)gr * gridDim.x;
+  bool requested = false;
+  // rows of X into the A1 tile (zeros past M)
+  auto request = [&](long long t) {
+    requested = true;
+    if (gt != 0) return;
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(mbar_x),
+                 "r"(kA1Bytes)
+                 : "memory");
+    const uint32_t dst = smem_u32(a1);
+#pragma unroll
+    for (int k = 0; k < kBoxes; ++k)
+      tma_load_2d(dst + k * kBoxBytes, &x_map, k * kBoxCols, (int)(t * kTcRows), mbar_x);
+    tma_load_2d(dst + kBoxes * kBoxBytes, &x_last, kBoxes * kBoxCols, (int)(t * kTcRows), mbar_x);
+  };
+  if (tid == 0) {
+    for (int k = 0; k < 2 * kTcGroups; ++k)
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(smem_u32(mbar + k)) : "memory");
+    asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+    fence_async_smem();
+  }
+  __syncthreads();
+  if (!FROM_MOM && tile < ntiles) request(tile);
 
   // ---- weights into the canonical layout; biases
   for (int c = tid; c < kMlpHidden * (kMlpIn / 8); c += kTcThreads) {
@@ -142,10 +221,6 @@ __global__ void __launch_bounds__(kTcThreads, 1)
   for (int c = tid; c < 2 * kMlpHidden + kMlpOut; c += kTcThreads)
     sb[c] = c < kMlpHidden ? p.b1[c] : (c < 2 * kMlpHidden ? p.b2[c - kMlpHidden]
                                                            : p.b3[c - 2 * kMlpHidden]);
-  if (tid == 0) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(mbar_a) : "memory");
-    asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
-  }
   if (warp == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(
                      smem_u32(tmem_slot)),
@@ -157,21 +232,30 @@ __global__ void __launch_bounds__(kTcThreads, 1)
   fence_before();
   __syncthreads();
   fence_after();
-  const uint32_t tmem = *tmem_slot;
+  const uint32_t tmem = *tmem_slot + kColGroup * gr;
   // TMEM lanes of this warp: 32 (warp % 4) ..
   const uint32_t lane_addr = tmem + ((uint32_t)(32 * (warp & 3)) << 16);
 
   const uint32_t sw1 = smem_u32(smem + kOffSW1), sw2 = smem_u32(smem + kOffSW2);
-  const uint32_t sw3 = smem_u32(smem + kOffSW3), sa1 = smem_u32(smem + kOffSA1);
-  const uint32_t sa2 = smem_u32(smem + kOffSA2), sa3 = smem_u32(smem + kOffSA3);
-  uint32_t phase = 0;
+  const uint32_t sw3 = smem_u32(smem + kOffSW3), sa1 = smem_u32(a1);
+  uint32_t phase = 0, xphase = 0;
   bool ok = true;
-  const long long ntiles = (M + kTcRows - 1) / kTcRows;
+  // the group's threads wait for the MMAs committed so far (the same decision in each)
+  auto sync_mma = [&]() {
+    ok = !group_any(gr, !mbar_wait(mbar_a, phase));
+    phase ^= 1;
+    fence_after();
+    return ok;
+  };
+  auto handoff = [&]() {  // the group's writes before the next MMAs
+    fence_before();
+    group_sync(gr);
+    fence_after();
+  };
 
-  for (long long tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x) {
+  for (; tile < ntiles; tile += stride) {
     const long long row = tile * kTcRows + r;
     const bool valid = row < M;
-    unsigned char *a1 = smem + kOffSA1;
     // ---- input rows
     if (FROM_MOM) {
       if (valid) {
@@ -181,91 +265,81 @@ __global__ void __launch_bounds__(kTcThreads, 1)
           *reinterpret_cast<uint4 *>(a1 + cm_offset(r, 8 * kb, kMlpIn)) =
               make_uint4(0u, 0u, 0u, 0u);
       }
+      fence_async_smem();
     } else {
-#pragma unroll 3
-      for (int kb = half * (kMlpIn / 16); kb < (half + 1) * (kMlpIn / 16); ++kb) {
-        const uint4 q = valid ? *reinterpret_cast<const uint4 *>(X + row * kMlpIn + 8 * kb)
-                              : make_uint4(0u, 0u, 0u, 0u);
-        *reinterpret_cast<uint4 *>(a1 + cm_offset(r, 8 * kb, kMlpIn)) = q;
-      }
+      ok = !group_any(gr, !mbar_wait(mbar_x, xphase));
+      if (!ok) break;
+      xphase ^= 1;
+      requested = false;
     }
-    fence_async_smem();
-    fence_before();
-    __syncthreads();
-    fence_after();
-    // ---- layer 1: D[128 x 64] (TMEM cols 0..63) = A1[128 x 288] W1^T
-    if (tid == 0) {
+    handoff();
+    // ---- layer 1: D[128 x 64] = A1[128 x 288] W1^T
+    if (gt == 0) {
 #pragma unroll 1
       for (int ks = 0; ks < kMlpIn / 16; ++ks)
-        umma(tmem, sdesc(sa1 + 256 * ks, 128, (kMlpIn / 8) * 128),
+        umma(tmem + kCol1,
+             FROM_MOM ? sdesc(sa1 + 256 * ks, 128, (kMlpIn / 8) * 128)
+                      : sdesc_swizzled(sa1 + (ks / 4) * kBoxBytes + 32 * (ks % 4), ks / 4 < kBoxes),
              sdesc(sw1 + 256 * ks, 128, (kMlpIn / 8) * 128), idesc_bf16(128, 64), ks > 0);
       umma_commit(mbar_a);
     }
-    ok = !__syncthreads_or(!mbar_wait(mbar_a, phase));  // same decision in every thread
-    phase ^= 1;
-    fence_after();
-    if (!ok) break;
-    hidden_epilogue<TRACE>(lane_addr + 0, sb, smem + kOffSA2, r, half,
+    if (!sync_mma()) break;
+    if (!FROM_MOM && tile + stride < ntiles) request(tile + stride);  // A1 has been read
+    hidden_epilogue<TRACE>(lane_addr + kCol1, sb, lane_addr + kColH + 16 * half, half,
                            TRACE && valid ? H + row * (2 * kMlpHidden) : nullptr);
-    fence_async_smem();
-    fence_before();
-    __syncthreads();
-    fence_after();
-    // ---- layer 2 (TMEM cols 64..127)
-    if (tid == 0) {
+    handoff();
+    // ---- layer 2
+    if (gt == 0) {
 #pragma unroll
       for (int ks = 0; ks < kMlpHidden / 16; ++ks)
-        umma(tmem + 64, sdesc(sa2 + 256 * ks, 128, (kMlpHidden / 8) * 128),
-             sdesc(sw2 + 256 * ks, 128, (kMlpHidden / 8) * 128), idesc_bf16(128, 64), ks > 0);
+        umma_ts(tmem + kCol2, tmem + kColH + 8 * ks,
+                sdesc(sw2 + 256 * ks, 128, (kMlpHidden / 8) * 128), idesc_bf16(128, 64), ks > 0);
       umma_commit(mbar_a);
     }
-    ok = !__syncthreads_or(!mbar_wait(mbar_a, phase));
-    phase ^= 1;
-    fence_after();
-    if (!ok) break;
-    hidden_epilogue<TRACE>(lane_addr + 64, sb + kMlpHidden, smem + kOffSA3, r, half,
+    if (!sync_mma()) break;
+    hidden_epilogue<TRACE>(lane_addr + kCol2, sb + kMlpHidden, lane_addr + kColH + 16 * half, half,
                            TRACE && valid ? H + row * (2 * kMlpHidden) + kMlpHidden : nullptr);
-    fence_async_smem();
-    fence_before();
-    __syncthreads();
-    fence_after();
-    // ---- layer 3 (TMEM cols 128..159): each half reads 16 of the 32 columns
-    if (tid == 0) {
+    handoff();
+    // ---- layer 3: each half reads 16 of the 32 columns
+    if (gt == 0) {
 #pragma unroll
       for (int ks = 0; ks < kMlpHidden / 16; ++ks)
-        umma(tmem + 128, sdesc(sa3 + 256 * ks, 128, (kMlpHidden / 8) * 128),
-             sdesc(sw3 + 256 * ks, 128, (kMlpHidden / 8) * 128), idesc_bf16(128, 32), ks > 0);
+        umma_ts(tmem + kCol1, tmem + kColH + 8 * ks,
+                sdesc(sw3 + 256 * ks, 128, (kMlpHidden / 8) * 128), idesc_bf16(128, 32), ks > 0);
       umma_commit(mbar_a);
     }
-    ok = !__syncthreads_or(!mbar_wait(mbar_a, phase));
-    phase ^= 1;
-    fence_after();
-    if (!ok) break;
+    if (!sync_mma()) break;
     float y[16];
-    tmem_ld16(lane_addr + 128 + 16 * half, y);
-    if (valid) {
-      const float *b3 = sb + 2 * kMlpHidden + 16 * half;
-      if (FROM_MOM) {
+    tmem_ld16(lane_addr + kCol1 + 16 * half, y);
+    const float *b3 = sb + 2 * kMlpHidden + 16 * half;
+    if (FROM_MOM) {
+      if (valid) {
 #pragma unroll
         for (int k = 0; k < 16; ++k)
           if (16 * half + k < kMlpOutUsed) Y[(16 * half + k) * M + row] = y[k] + b3[k];
-      } else {
+      }
+    } else {
 #pragma unroll
-        for (int k = 0; k < 16; k += 4)
-          *reinterpret_cast<float4 *>(Y + row * kMlpOut + 16 * half + k) =
-              make_float4(y[k] + b3[k], y[k + 1] + b3[k + 1], y[k + 2] + b3[k + 2],
-                          y[k + 3] + b3[k + 3]);
+      for (int k = 0; k < 16; ++k) ys[r * kYRow + 16 * half + k] = y[k] + b3[k];
+      group_sync(gr);
+      const long long row0 = tile * kTcRows;
+      const int lane = tid & 31;
+#pragma unroll
+      for (int k = 0; k < kTcRows; k += kGroupThreads / 32) {
+        const int q = k + gt / 32;
+        if (row0 + q < M) Y[(row0 + q) * kMlpOut + lane] = ys[q * kYRow + lane];
       }
     }
+    // the accumulators and, over the next tile's barriers, ys have been read
     fence_before();
-    __syncthreads();  // the next tile overwrites A1 and the accumulators
-    fence_after();
   }
 
   if (!ok) {
-    if (tid == 0) atomicExch(status, 1);
-    // let any MMA still in flight finish before the memory goes away
-    mbar_wait(mbar_a, phase);
+    if (gt == 0) atomicExch(status, 1);
+    // let copies and MMAs still in flight finish before the memory goes away
+    // (at the last phase waited for)
+    if (requested) mbar_wait(mbar_x, xphase);
+    mbar_wait(mbar_a, phase ^ 1);
   }
   fence_before();
   __syncthreads();
@@ -278,6 +352,19 @@ __global__ void __launch_bounds__(kTcThreads, 1)
 
 }  // namespace
 
+// boxes of kTcRows rows of X [M][288] and cols columns
+static cudaError_t row_map(const void *X, long long M, int cols, CUtensorMapSwizzle swizzle,
+                           CUtensorMap *map) {
+  PFN_cuTensorMapEncodeTiled_v12000 encode = tensor_map_encoder();
+  if (!encode) return cudaErrorNotSupported;
+  const cuuint64_t dims[2] = {kMlpIn, (cuuint64_t)M}, strides[1] = {kMlpIn * 2};
+  const cuuint32_t box[2] = {(cuuint32_t)cols, kTcRows}, estr[2] = {1, 1};
+  const CUresult r = encode(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void *>(X), dims,
+                            strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle,
+                            CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
+}
+
 cudaError_t launch_mlp_tc(const MlpDevice &p, const void *X, const float *mom, const Grid *g,
                           long long M, float *Y, int *status, int nblocks, cudaStream_t st,
                           float *H) {
@@ -288,11 +375,16 @@ cudaError_t launch_mlp_tc(const MlpDevice &p, const void *X, const float *mom, c
   cudaError_t e =
       cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTcSmem);
   if (e != cudaSuccess) return e;
+  CUtensorMap map{}, last{};
+  if (!from_mom) {
+    e = row_map(X, M, kBoxCols, CU_TENSOR_MAP_SWIZZLE_128B, &map);
+    if (e == cudaSuccess) e = row_map(X, M, kLastCols, CU_TENSOR_MAP_SWIZZLE_64B, &last);
+    if (e != cudaSuccess) return e;
+  }
   const long long tiles = (M + kTcRows - 1) / kTcRows;
   const int nb = (int)(tiles < nblocks ? tiles : nblocks);
   const Grid gg = g ? *g : Grid{1, 1, 1, M};
-  kern<<<nb, kTcThreads, kTcSmem, st>>>(p, static_cast<const __nv_bfloat16 *>(X), mom, gg, M, Y,
-                                        status, H);
+  kern<<<nb, kTcThreads, kTcSmem, st>>>(p, map, last, mom, gg, M, Y, status, H);
   return cudaGetLastError();
 }
 
