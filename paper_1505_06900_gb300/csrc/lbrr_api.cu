@@ -644,9 +644,8 @@ void lb_mlp_destroy(lb_mlp *m) {
   if (!m) return;
   DeviceGuard dg(m->device);
   if (m->stream) cudaStreamSynchronize(m->stream);
-  void *bufs[] = {m->d.params, m->d.adam_m, m->d.adam_v, m->d.w1,    m->d.w2,
-                  m->d.w3,     m->d.w2t,    m->d.w3t,    m->scaling, m->gpart,
-                  m->lpart,    m->dloss,    m->status};
+  void *bufs[] = {m->d.params, m->d.adam_m, m->d.adam_v, m->d.w1,  m->scaling,
+                  m->gpart,    m->lpart,    m->dloss,    m->status};
   for (void *b : bufs)
     if (b) cudaFree(b);
   delete m;
@@ -669,11 +668,7 @@ int lb_mlp_create(lb_mlp **out) {
   e = cudaMalloc(&m->d.params, 4 * P);
   if (e == cudaSuccess) e = cudaMalloc(&m->d.adam_m, 4 * P);
   if (e == cudaSuccess) e = cudaMalloc(&m->d.adam_v, 4 * P);
-  if (e == cudaSuccess) e = cudaMalloc(&m->d.w1, 2 * lbrr::kMlpHidden * lbrr::kMlpIn);
-  if (e == cudaSuccess) e = cudaMalloc(&m->d.w2, 2 * lbrr::kMlpHidden * lbrr::kMlpHidden);
-  if (e == cudaSuccess) e = cudaMalloc(&m->d.w3, 2 * lbrr::kMlpOut * lbrr::kMlpHidden);
-  if (e == cudaSuccess) e = cudaMalloc(&m->d.w2t, 2 * lbrr::kMlpHidden * lbrr::kMlpHidden);
-  if (e == cudaSuccess) e = cudaMalloc(&m->d.w3t, 2 * lbrr::kMlpOut * lbrr::kMlpHidden);
+  if (e == cudaSuccess) e = cudaMalloc(&m->d.w1, lbrr::kMlpWeightBytes);
   if (e == cudaSuccess) e = cudaMalloc(&m->scaling, 4 * 37);
   if (e == cudaSuccess) e = cudaMalloc(&m->gpart, 4 * P * (size_t)m->nblocks);
   if (e == cudaSuccess) e = cudaMalloc(&m->lpart, 4 * (size_t)m->nblocks);
@@ -685,6 +680,10 @@ int lb_mlp_create(lb_mlp **out) {
     lb_mlp_destroy(m);
     return fail(nullptr, LB_ENOMEM, "cannot allocate the network");
   }
+  m->d.w2 = m->d.w1 + lbrr::kMlpW1Bytes / 2;
+  m->d.w3 = m->d.w2 + lbrr::kMlpW2Bytes / 2;
+  m->d.w2t = m->d.w3 + lbrr::kMlpW3Bytes / 2;
+  m->d.w3t = m->d.w2t + lbrr::kMlpW2Bytes / 2;
   m->d.b1 = m->d.params + lbrr::kOffB1;
   m->d.b2 = m->d.params + lbrr::kOffB2;
   m->d.b3 = m->d.params + lbrr::kOffB3;

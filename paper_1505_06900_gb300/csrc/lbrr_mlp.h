@@ -27,10 +27,17 @@ constexpr int kOffW3 = kOffB2 + kMlpHidden;
 constexpr int kOffB3 = kOffW3 + kMlpOut * kMlpHidden;
 constexpr int kMlpParams = kOffB3 + kMlpOut;  // 24736
 
+// Bytes of the BF16 copies of the weights, and of all five.
+constexpr uint32_t kMlpW1Bytes = kMlpHidden * kMlpIn * 2, kMlpW2Bytes = kMlpHidden * kMlpHidden * 2,
+                   kMlpW3Bytes = kMlpOut * kMlpHidden * 2;
+constexpr uint32_t kMlpWeightBytes = kMlpW1Bytes + 2 * kMlpW2Bytes + 2 * kMlpW3Bytes;
+
 // Device view of one network: FP32 master parameters and Adam moments, BF16
-// copies of the weights in K-major layout (row = output unit) for the forward
-// products and transposed copies of W2 and W3 for the backward products, and
-// the feature / target standardisation.
+// copies of the weights (row = output unit) for the forward products and
+// transposed copies of W2 and W3 for the backward products, and the feature /
+// target standardisation. The copies lie one after another from w1, each in the
+// order in which the products take it from shared memory (cm_offset of
+// lbrr_tc.cuh), so that one bulk copy brings a block all it needs.
 struct MlpDevice {
   float *params, *adam_m, *adam_v;
   __nv_bfloat16 *w1, *w2, *w3, *w2t, *w3t;
@@ -187,6 +194,9 @@ cudaError_t launch_step_targets(const MlpDevice &p, const float *fpre, int ppre,
                                 cudaStream_t st);
 // cuTensorMapEncodeTiled, or null where the driver has none.
 PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder();
+// TMA map of X [M][288] (BF16) in boxes of 128 rows and cols columns.
+cudaError_t make_row_map(const void *X, long long M, int cols, CUtensorMapSwizzle swizzle,
+                         CUtensorMap *map);
 // Network forward on the tcgen05 tensor cores (lbrr_mlp_tc.cu). With mom:
 // rows are the cells of grid *g, features from the moment field, outputs the
 // 17 standardised predictions Y [17][N]. Without: rows X [M][288] BF16, Y

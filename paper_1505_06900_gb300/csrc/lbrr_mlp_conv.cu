@@ -106,8 +106,8 @@ constexpr uint32_t kTmemCols = 512;
 
 constexpr uint32_t kSmW1 = 0;
 constexpr uint32_t kSmW2 = kSmW1 + kMmas1 * kW1Bytes;
-constexpr uint32_t kSmW3 = kSmW2 + kMlpHidden * kMlpHidden * 2;
-constexpr uint32_t kOffA1 = kSmW3 + kMlpOut * kMlpHidden * 2;
+constexpr uint32_t kSmW3 = kSmW2 + kMlpW2Bytes;
+constexpr uint32_t kOffA1 = kSmW3 + kMlpW3Bytes;
 constexpr uint32_t kOffPop = kOffA1 + kStages * kStageBytes;
 constexpr uint32_t kOffMisc = kOffPop + kGroups * kPopBytes;
 constexpr uint32_t kOffBias = 512;                   // biases, after barriers and counters
@@ -134,10 +134,6 @@ static_assert(kNumBars * 8 + 8 + 4 * (1 + kIssuers) <= kOffBias,
 
 __device__ __forceinline__ void mbar_arrive(uint32_t mbar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(mbar) : "memory");
-}
-__device__ __forceinline__ void mbar_expect_tx(uint32_t mbar, uint32_t bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(mbar), "r"(bytes)
-               : "memory");
 }
 // 3-D and 5-D tiled TMA loads (coordinates innermost first), completing on mbar
 __device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap *map, int c0, int c1,
@@ -252,7 +248,7 @@ __global__ void __launch_bounds__(kConvThreads, 1)
         nb = k < 6 ? (k >> 1) + 3 * r9 : -1;
         ch = 8 + (k & 1);
       }
-      w[k] = nb >= 0 ? __bfloat16_as_ushort(p.w1[n * kMlpIn + kMlpMoments * nb + ch]) : 0;
+      w[k] = nb >= 0 ? __bfloat16_as_ushort(p.w1[cm_offset(n, kMlpMoments * nb + ch, kMlpIn) / 2]) : 0;
     }
     if (kind == 1 && h == 1 && r9 == 4) {  // b1 = b_hi + b_lo on the constant inputs
       const __nv_bfloat16 hi = __float2bfloat16_rn(p.b1[n]);
@@ -268,16 +264,8 @@ __global__ void __launch_bounds__(kConvThreads, 1)
         make_uint4(w[0] | ((uint32_t)w[1] << 16), w[2] | ((uint32_t)w[3] << 16),
                    w[4] | ((uint32_t)w[5] << 16), w[6] | ((uint32_t)w[7] << 16));
   }
-  for (int c = tid; c < kMlpHidden * (kMlpHidden / 8); c += kConvThreads) {
-    const int n = c / (kMlpHidden / 8), kb = c - n * (kMlpHidden / 8);
-    *reinterpret_cast<uint4 *>(smem + kSmW2 + cm_offset(n, 8 * kb, kMlpHidden)) =
-        *reinterpret_cast<const uint4 *>(p.w2 + n * kMlpHidden + 8 * kb);
-  }
-  for (int c = tid; c < kMlpOut * (kMlpHidden / 8); c += kConvThreads) {
-    const int n = c / (kMlpHidden / 8), kb = c - n * (kMlpHidden / 8);
-    *reinterpret_cast<uint4 *>(smem + kSmW3 + cm_offset(n, 8 * kb, kMlpHidden)) =
-        *reinterpret_cast<const uint4 *>(p.w3 + n * kMlpHidden + 8 * kb);
-  }
+  for (int c = tid; c < (int)(kMlpW2Bytes + kMlpW3Bytes) / 16; c += kConvThreads)
+    reinterpret_cast<uint4 *>(smem + kSmW2)[c] = reinterpret_cast<const uint4 *>(p.w2)[c];
   for (int c = tid; c < 2 * kMlpHidden + kMlpOut + kMlpOutUsed; c += kConvThreads)
     sb[c] = c < kMlpHidden ? p.b1[c]
             : c < 2 * kMlpHidden ? p.b2[c - kMlpHidden]

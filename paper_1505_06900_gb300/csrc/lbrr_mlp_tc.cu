@@ -8,9 +8,9 @@
 // canonical K-major layout without swizzle: 8 x 8 "core matrices" of 128
 // contiguous bytes (8 rows of 16 bytes), adjacent core matrices along K 128
 // bytes apart (leading byte offset) and adjacent 8-row groups K/8 * 128 bytes
-// apart (stride byte offset). A tile's 128 input rows come by TMA in boxes of 64
-// columns in the layout with 128-byte swizzle, the last 32 with 64-byte swizzle;
-// one thread of the group issues the MMAs of a layer (M = 128, N = 64, 64, 32)
+// apart (stride byte offset), as they lie in memory. A tile's 128 input rows
+// come by TMA in boxes of 64 columns in the layout with 128-byte swizzle, the
+// last 32 with 64-byte swizzle; one thread of the group issues the MMAs of a layer (M = 128, N = 64, 64, 32)
 // and commits them to the group's mbarrier; the threads, two to a row (TMEM
 // lane), then read the accumulator (tcgen05.ld 32x32b), add the bias, apply
 // tanh and write the BF16 row back into TMEM (tcgen05.st), the A operand of the
@@ -51,16 +51,13 @@ constexpr uint32_t kColGroup = 192, kCol1 = 0, kCol2 = 64, kColH = 128;
 constexpr uint32_t kTmemCols = 512;
 
 // shared-memory plan (bytes, all 1024-aligned up to the output rows)
-constexpr uint32_t kW1Bytes = kMlpHidden * kMlpIn * 2;        // 36864
-constexpr uint32_t kW2Bytes = kMlpHidden * kMlpHidden * 2;    // 8192
-constexpr uint32_t kW3Bytes = kMlpOut * kMlpHidden * 2;       // 4096
 constexpr uint32_t kA1Bytes = kTcRows * kMlpIn * 2;           // 73728
 constexpr int kYRow = kMlpOut + 1;                            // odd: no bank conflicts
 constexpr uint32_t kYBytes = kTcRows * kYRow * 4;             // 16896
 constexpr uint32_t kOffSW1 = 0;
-constexpr uint32_t kOffSW2 = kOffSW1 + kW1Bytes;
-constexpr uint32_t kOffSW3 = kOffSW2 + kW2Bytes;
-constexpr uint32_t kOffSA1 = kOffSW3 + kW3Bytes;
+constexpr uint32_t kOffSW2 = kOffSW1 + kMlpW1Bytes;
+constexpr uint32_t kOffSW3 = kOffSW2 + kMlpW2Bytes;
+constexpr uint32_t kOffSA1 = kOffSW3 + kMlpW3Bytes;
 constexpr uint32_t kOffY = kOffSA1 + kTcGroups * kA1Bytes;
 constexpr uint32_t kOffMisc = kOffY + kTcGroups * kYBytes;  // mbarriers, TMEM address, biases
 constexpr uint32_t kTcSmem = kOffMisc + 1024;
@@ -69,22 +66,6 @@ constexpr int kBoxCols = 64, kBoxes = kMlpIn / kBoxCols, kLastCols = kMlpIn - kB
 constexpr uint32_t kBoxBytes = kTcRows * kBoxCols * 2;
 static_assert(kLastCols == 32, "64-byte rows");
 static_assert(kOffSA1 % 1024 == 0 && kA1Bytes % 1024 == 0, "swizzle atoms");
-
-// Descriptor of a K-major operand with swizzled rows of 128 or 64 bytes (8 rows
-// an atom, atoms contiguous); a K step of 16 columns moves its start address.
-__device__ __forceinline__ uint64_t sdesc_swizzled(uint32_t saddr, bool wide) {
-  return sdesc(saddr, 16, wide ? 1024 : 512) | ((uint64_t)(wide ? 2 : 4) << 61);
-}
-// 2-D tiled TMA load, completing on mbar
-__device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap *map, int c0, int c1,
-                                            uint32_t mbar) {
-  asm volatile(
-      "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
-      " [%0], [%1, {%2, %3}], [%4];\n" ::"r"(dst),
-      "l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(c1), "r"(mbar)
-      : "memory");
-}
-static_assert(kTcSmem <= 232448, "fits the shared memory of one block");
 
 __device__ __forceinline__ void group_sync(int g) {
   asm volatile("bar.sync %0, %1;\n" ::"r"(1 + g), "n"(kGroupThreads) : "memory");
@@ -168,9 +149,9 @@ __global__ void __launch_bounds__(kTcThreads, 1)
   const int tid = threadIdx.x, warp = tid >> 5;
   const int gr = tid / kGroupThreads, gt = tid % kGroupThreads;
   const int r = gt & (kTcRows - 1), half = gt >> 7;  // row, and which half of its work
-  // of each group: MMAs done, rows landed
+  // of each group: MMAs done, rows landed; then the weights landed
   uint64_t *mbar = reinterpret_cast<uint64_t *>(smem + kOffMisc);
-  uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(smem + kOffMisc + 16 * kTcGroups);
+  uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(smem + kOffMisc + 16 * kTcGroups + 8);
   float *sb = reinterpret_cast<float *>(smem + kOffMisc + 64);  // b1, b2, b3 (160)
   unsigned char *a1 = smem + kOffSA1 + gr * kA1Bytes;
   float *ys = reinterpret_cast<float *>(smem + kOffY + gr * kYBytes);
@@ -184,40 +165,24 @@ __global__ void __launch_bounds__(kTcThreads, 1)
   auto request = [&](long long t) {
     requested = true;
     if (gt != 0) return;
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(mbar_x),
-                 "r"(kA1Bytes)
-                 : "memory");
+    mbar_expect_tx(mbar_x, kA1Bytes);
     const uint32_t dst = smem_u32(a1);
 #pragma unroll
     for (int k = 0; k < kBoxes; ++k)
       tma_load_2d(dst + k * kBoxBytes, &x_map, k * kBoxCols, (int)(t * kTcRows), mbar_x);
     tma_load_2d(dst + kBoxes * kBoxBytes, &x_last, kBoxes * kBoxCols, (int)(t * kTcRows), mbar_x);
   };
+  const uint32_t mbar_w = smem_u32(mbar + 2 * kTcGroups);
   if (tid == 0) {
-    for (int k = 0; k < 2 * kTcGroups; ++k)
-      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(smem_u32(mbar + k)) : "memory");
+    for (int k = 0; k <= 2 * kTcGroups; ++k) mbar_init(smem_u32(mbar + k), 1);
     asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
     fence_async_smem();
+    mbar_expect_tx(mbar_w, kOffSA1);
+    bulk_load(smem_u32(smem), p.w1, kOffSA1, mbar_w);
   }
   __syncthreads();
   if (!FROM_MOM && tile < ntiles) request(tile);
-
-  // ---- weights into the canonical layout; biases
-  for (int c = tid; c < kMlpHidden * (kMlpIn / 8); c += kTcThreads) {
-    const int n = c / (kMlpIn / 8), kb = c - n * (kMlpIn / 8);
-    *reinterpret_cast<uint4 *>(smem + kOffSW1 + cm_offset(n, 8 * kb, kMlpIn)) =
-        *reinterpret_cast<const uint4 *>(p.w1 + n * kMlpIn + 8 * kb);
-  }
-  for (int c = tid; c < kMlpHidden * (kMlpHidden / 8); c += kTcThreads) {
-    const int n = c / (kMlpHidden / 8), kb = c - n * (kMlpHidden / 8);
-    *reinterpret_cast<uint4 *>(smem + kOffSW2 + cm_offset(n, 8 * kb, kMlpHidden)) =
-        *reinterpret_cast<const uint4 *>(p.w2 + n * kMlpHidden + 8 * kb);
-  }
-  for (int c = tid; c < kMlpOut * (kMlpHidden / 8); c += kTcThreads) {
-    const int n = c / (kMlpHidden / 8), kb = c - n * (kMlpHidden / 8);
-    *reinterpret_cast<uint4 *>(smem + kOffSW3 + cm_offset(n, 8 * kb, kMlpHidden)) =
-        *reinterpret_cast<const uint4 *>(p.w3 + n * kMlpHidden + 8 * kb);
-  }
+  // ---- biases
   for (int c = tid; c < 2 * kMlpHidden + kMlpOut; c += kTcThreads)
     sb[c] = c < kMlpHidden ? p.b1[c] : (c < 2 * kMlpHidden ? p.b2[c - kMlpHidden]
                                                            : p.b3[c - 2 * kMlpHidden]);
@@ -253,7 +218,8 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     fence_after();
   };
 
-  for (; tile < ntiles; tile += stride) {
+  ok = !group_any(gr, !mbar_wait(mbar_w, 0));
+  for (; tile < ntiles && ok; tile += stride) {
     const long long row = tile * kTcRows + r;
     const bool valid = row < M;
     // ---- input rows
@@ -279,7 +245,8 @@ __global__ void __launch_bounds__(kTcThreads, 1)
       for (int ks = 0; ks < kMlpIn / 16; ++ks)
         umma(tmem + kCol1,
              FROM_MOM ? sdesc(sa1 + 256 * ks, 128, (kMlpIn / 8) * 128)
-                      : sdesc_swizzled(sa1 + (ks / 4) * kBoxBytes + 32 * (ks % 4), ks / 4 < kBoxes),
+                      : sdesc_swizzled(sa1 + (ks / 4) * kBoxBytes + 32 * (ks % 4), 16,
+                                       ks / 4 < kBoxes ? 1024 : 512, ks / 4 < kBoxes),
              sdesc(sw1 + 256 * ks, 128, (kMlpIn / 8) * 128), idesc_bf16(128, 64), ks > 0);
       umma_commit(mbar_a);
     }
@@ -338,6 +305,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     if (gt == 0) atomicExch(status, 1);
     // let copies and MMAs still in flight finish before the memory goes away
     // (at the last phase waited for)
+    mbar_wait(mbar_w, 0);
     if (requested) mbar_wait(mbar_x, xphase);
     mbar_wait(mbar_a, phase ^ 1);
   }
@@ -352,9 +320,8 @@ __global__ void __launch_bounds__(kTcThreads, 1)
 
 }  // namespace
 
-// boxes of kTcRows rows of X [M][288] and cols columns
-static cudaError_t row_map(const void *X, long long M, int cols, CUtensorMapSwizzle swizzle,
-                           CUtensorMap *map) {
+cudaError_t make_row_map(const void *X, long long M, int cols, CUtensorMapSwizzle swizzle,
+                         CUtensorMap *map) {
   PFN_cuTensorMapEncodeTiled_v12000 encode = tensor_map_encoder();
   if (!encode) return cudaErrorNotSupported;
   const cuuint64_t dims[2] = {kMlpIn, (cuuint64_t)M}, strides[1] = {kMlpIn * 2};
@@ -377,8 +344,8 @@ cudaError_t launch_mlp_tc(const MlpDevice &p, const void *X, const float *mom, c
   if (e != cudaSuccess) return e;
   CUtensorMap map{}, last{};
   if (!from_mom) {
-    e = row_map(X, M, kBoxCols, CU_TENSOR_MAP_SWIZZLE_128B, &map);
-    if (e == cudaSuccess) e = row_map(X, M, kLastCols, CU_TENSOR_MAP_SWIZZLE_64B, &last);
+    e = make_row_map(X, M, kBoxCols, CU_TENSOR_MAP_SWIZZLE_128B, &map);
+    if (e == cudaSuccess) e = make_row_map(X, M, kLastCols, CU_TENSOR_MAP_SWIZZLE_64B, &last);
     if (e != cudaSuccess) return e;
   }
   const long long tiles = (M + kTcRows - 1) / kTcRows;
