@@ -87,6 +87,13 @@ bool tiled16_supported(const Grid &g);
 cudaError_t launch_step_tiled16_odd(int q, int storage, int model, void *f, const Grid &g,
                                     float om1, cudaStream_t st);
 
+// An update of a 16-bit store, two cells per thread (lbrr_words16.cu); usable
+// when words16_supported(q, g, parity) (parity 0: an even number of cells,
+// parity 1: rows of an even number; no small stores).
+bool words16_supported(int q, const Grid &g, int parity);
+cudaError_t launch_step_words16(int q, int storage, int model, void *f, const Grid &g, float om1,
+                                int parity, cudaStream_t st);
+
 // f = f0 + f1 (mode 1) or f0 (mode 0) from device fields rho [N], u [D][N].
 cudaError_t launch_init(int q, int storage, int model, void *f, const Grid &g, const float *rho,
                         const float *u, float tau, int mode, cudaStream_t st);
