@@ -5,6 +5,7 @@
 // (the weights and the transposed copies of W2 and W3).
 #include <cstdint>
 
+#include "lbrr_chain.cuh"
 #include "lbrr_launch.h"
 #include "lbrr_mlp.h"
 #include "lbrr_act.cuh"
@@ -22,11 +23,12 @@ constexpr int kReduce = 64;
 // Sum of the block partials (fixed order), optional Adam update of the FP32
 // master parameters and refresh of the BF16 copies; nothing when the
 // training kernel recorded a timeout (its partials are incomplete).
-__global__ void mlp_reduce_adam_kernel(MlpDevice p, const float *__restrict__ gpart, int nparts,
-                                       float *__restrict__ grad_out, int adam, float lr,
+__global__ void mlp_reduce_adam_kernel(MlpDevice p, const float *gpart, int nparts,
+                                       float *grad_out, int adam, float lr,
                                        float bc1, float bc2, const int *status) {
   const int k = blockIdx.x * blockDim.x + threadIdx.x;
   if (k >= kMlpParams) return;
+  chain_wait();
   const int timed_out = *status;
   const float m0 = adam ? p.adam_m[k] : 0.f, v0 = adam ? p.adam_v[k] : 0.f;
   const float w0 = adam ? p.params[k] : 0.f;
@@ -80,9 +82,9 @@ __device__ void mlp_refresh_one(MlpDevice p, int k, float w) {
 cudaError_t launch_mlp_reduce(const MlpDevice &p, const float *gpart, int nparts, float *grad_out,
                               int adam, float lr, float bc1, float bc2, const float *lpart,
                               double *loss_out, const int *status, cudaStream_t st) {
-  mlp_reduce_adam_kernel<<<(kMlpParams + kReduce - 1) / kReduce, kReduce, 0, st>>>(
-      p, gpart, nparts, grad_out, adam, lr, bc1, bc2, status);
-  cudaError_t e = cudaGetLastError();
+  const cudaError_t e =
+      launch_chained(mlp_reduce_adam_kernel, (kMlpParams + kReduce - 1) / kReduce, kReduce, 0, st,
+                     p, gpart, nparts, grad_out, adam, lr, bc1, bc2, status);
   if (e != cudaSuccess || !loss_out) return e;
   loss_sum_kernel<<<1, 32, 0, st>>>(lpart, nparts, loss_out);
   return cudaGetLastError();

@@ -31,9 +31,9 @@
 // further on; it is copied by one load per half of 17 chunks. The tile rows that
 // fall on the padding (8 of 72 positions at nx = 64) are computed and dropped,
 // and the rest of b1 meets the constant inputs of the row after the centre, so
-// that the bias is b1 to the bit. 64^3 takes 42 us a step; the moment
+// that the bias is b1 to the bit. 64^3 takes 34 us a step; the moment
 // field, the network fed by threads (mlp_tc_kernel, one tile after another) and
-// the separate update, 119 (250^3: 1.42 and 6.91 ms).
+// the separate update, 119 (250^3: 1.41 and 6.91 ms).
 //
 // One persistent block per SM, nineteen warps:
 //   warp 0      TMA producer: per tile 2 tile loads (halves) for each of the 3 z
@@ -68,6 +68,7 @@
 
 #include <cstdint>
 
+#include "lbrr_chain.cuh"
 #include "lbrr_launch.h"
 #include "lbrr_mlp.h"
 #include "lbrr_act.cuh"
@@ -217,9 +218,8 @@ __device__ __forceinline__ void load_acc32(uint32_t taddr, uint32_t (&v)[32]) {
 template <int PARITY, typename IDX, bool TRACE = false, bool FLAT = false>
 __global__ void __launch_bounds__(kConvThreads, 1)
     mlp_conv_kernel(MlpDevice p, const __grid_constant__ CUtensorMap xs_map, const Grid g,
-                    float *__restrict__ f, const float om1, unsigned long long *fallbacks,
-                    const float bound, const float dead_zone, int *status,
-                    float *__restrict__ trace) {
+                    float *f, const float om1, unsigned long long *fallbacks, const float bound,
+                    const float dead_zone, int *status, float *trace) {
   extern __shared__ __align__(1024) unsigned char smem[];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   uint64_t *bars = reinterpret_cast<uint64_t *>(smem + kOffMisc);
@@ -289,6 +289,7 @@ __global__ void __launch_bounds__(kConvThreads, 1)
   fence_before();
   __syncthreads();
   fence_after();
+  chain_wait();  // the feature source is complete; the weights were before it began
   const uint32_t tmem = *tmem_slot;
   const uint32_t lim = wait_limit(status);
   // tiles of a row, or of a plane
@@ -548,8 +549,8 @@ __global__ void __launch_bounds__(kConvThreads, 1)
 constexpr int kFsThreads = 256, kFsOut = kFsThreads - 2;
 
 __global__ void __launch_bounds__(kFsThreads)
-    feature_source_kernel(MlpDevice p, const float *__restrict__ f, const Grid g, const int parity,
-                          uint4 *__restrict__ xs) {
+    feature_source_kernel(MlpDevice p, const float *f, const Grid g, const int parity, uint4 *xs) {
+  chain_wait();
   __shared__ uint32_t s89[kFsThreads];
   const long long px = g.nx + 2, py = g.ny + 2, pz = g.nz + 2, total = px * py * pz;
   const long long q = (long long)blockIdx.x * kFsOut + threadIdx.x - 1;
@@ -603,9 +604,8 @@ bool mlp_conv_rows(const Grid &g) { return g.nx % kCRows == 0 && g.walls == 0; }
 // Rows of whole tiles, and other grids whose padding is small enough for the
 // feature source to take no more memory than the predictions (17 floats a
 // cell) of the separate network, as it is where no extent is below 14. Times of
-// a step, this and the separate network: 14^3 18.5 and 22.0 us, 24 x 12 x 12
-// 18.5 and 20.9, 30^3 18.6 and 30.4, 96^3 106 and 406, 160 x 100 x 90 155 and
-// 660.
+// a step, this and the separate network: 14^3 8.9 and 22.0 us, 24 x 12 x 12 9.0
+// and 20.9, 30^3 12.3 and 30.4, 96^3 100 and 406, 160 x 100 x 90 150 and 660.
 bool mlp_conv_supported(const Grid &g) {
   return mlp_conv_rows(g) || (g.walls == 0 && feature_source_bytes(g) <= 68 * (size_t)g.n);
 }
@@ -657,8 +657,15 @@ cudaError_t make_feature_map(void *xs, const Grid &g, CUtensorMap *map) {
 cudaError_t launch_feature_source(const MlpDevice &p, const float *f, const Grid &g, int parity,
                                   void *xs, cudaStream_t st) {
   const long long cells = (long long)(g.nx + 2) * (g.ny + 2) * (g.nz + 2);
-  feature_source_kernel<<<(unsigned)((cells + kFsOut - 1) / kFsOut), kFsThreads, 0, st>>>(
-      p, f, g, parity, static_cast<uint4 *>(xs));
+  const unsigned blocks = (unsigned)((cells + kFsOut - 1) / kFsOut);
+  // Chained to the update before it where launches count. us a step, with and
+  // without: 16^3 9.0 and 10.5, 64^3 33.9 and 35.1, 128 x 64 x 64 53.2 and 53.5,
+  // but 96^3 101 and 100, 256^3 1493 and 1386. (With neither kernel chained 16^3
+  // takes 14.4, 64^3 38.6, 96^3 104, 256^3 1391.)
+  if (g.n <= 1 << 19)
+    return launch_chained(feature_source_kernel, blocks, kFsThreads, 0, st, p, f, g, parity,
+                          static_cast<uint4 *>(xs));
+  feature_source_kernel<<<blocks, kFsThreads, 0, st>>>(p, f, g, parity, static_cast<uint4 *>(xs));
   return cudaGetLastError();
 }
 
@@ -694,9 +701,8 @@ cudaError_t launch_mlp_conv_step(const MlpDevice &p, const CUtensorMap &map, con
   if (tiles >= (1LL << 31)) return cudaErrorInvalidValue;
   const int nb = (int)(tiles < nblocks ? tiles : nblocks);
   if (nb < 1) return cudaSuccess;
-  kern<<<nb, kConvThreads, kConvSmem, st>>>(p, map, g, f, om1, fallbacks, bound, dead_zone,
-                                            status, trace);
-  return cudaGetLastError();
+  return launch_chained(kern, nb, kConvThreads, kConvSmem, st, p, map, g, f, om1, fallbacks, bound,
+                        dead_zone, status, trace);
 }
 
 }  // namespace lbrr

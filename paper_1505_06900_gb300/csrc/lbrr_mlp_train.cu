@@ -39,6 +39,7 @@
 // 384, then h2 in FP32, then dh2 W2; layer 3 at 448, then dy W3.
 #include <cstdint>
 
+#include "lbrr_chain.cuh"
 #include "lbrr_launch.h"
 #include "lbrr_mlp.h"
 #include "lbrr_act.cuh"
@@ -154,8 +155,8 @@ __device__ __forceinline__ void warp_col_sums(float (&v)[N], float *dst, int lan
 template <bool TRACE>
 __global__ void __launch_bounds__(kThreads, 1)
     mlp_train_tc_kernel(MlpDevice p, const __grid_constant__ CUtensorMap x_map,
-                        const float *__restrict__ T, long long M, float *__restrict__ gpart,
-                        float *__restrict__ lpart, int *status, float *__restrict__ trace) {
+                        const float *T, long long M, float *gpart, float *lpart, int *status,
+                        float *trace) {
   extern __shared__ __align__(1024) unsigned char smem[];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int r = tid & (kRows - 1), half = tid >> 7;
@@ -181,6 +182,16 @@ __global__ void __launch_bounds__(kThreads, 1)
     for (int k = 0; k < 4; ++k) mbar_init(smem_u32(mbar + k), 1);
     asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
     fence_async_smem();
+  }
+  if (warp == 0) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(
+                     smem_u32(tmem_slot)),
+                 "r"(kTmemCols)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n" ::: "memory");
+  }
+  chain_wait();
+  if (tid == 0) {
     request(blockIdx.x);  // the launcher starts no block without a tile
     mbar_expect_tx(mbar_w, kMlpWeightBytes);
     bulk_load(smem_u32(smem + kSmW1), p.w1, kMlpWeightBytes, mbar_w);
@@ -191,13 +202,6 @@ __global__ void __launch_bounds__(kThreads, 1)
   for (int c = tid; c < 8 * kGbCols; c += kThreads)
     reinterpret_cast<float *>(smem + kSmGbw)[c] = 0.f;
   if (tid < 8) lossw[tid] = 0.f;
-  if (warp == 0) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(
-                     smem_u32(tmem_slot)),
-                 "r"(kTmemCols)
-                 : "memory");
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n" ::: "memory");
-  }
   fence_async_smem();
   fence_before();
   __syncthreads();
@@ -466,8 +470,8 @@ cudaError_t launch_mlp_train(const MlpDevice &p, const void *X, const float *T, 
   CUtensorMap map;
   e = make_row_map(X, M, kBoxCols, CU_TENSOR_MAP_SWIZZLE_128B, &map);
   if (e != cudaSuccess) return e;
-  kern<<<nb, kThreads, kTrainSmem, st>>>(p, map, T, M, gpart, lpart, status, trace);
-  return cudaGetLastError();
+  return launch_chained(kern, nb, kThreads, kTrainSmem, st, p, map, T, M, gpart, lpart, status,
+                        trace);
 }
 
 }  // namespace lbrr

@@ -21,6 +21,7 @@
 // 4096x3000 134 / 75.7 (20 updates). The tile kernel issues in 39% of its
 // slots: its phases (collision, exchange, sums) follow one another in all warps
 // of a block, and one block fills an SM's registers.
+#include "lbrr_chain.cuh"
 #include "lbrr_two.cuh"
 
 namespace lbrr {
@@ -57,8 +58,7 @@ struct Pass2 {
 // collision more.
 template <class B, int KIND>
 __global__ void __launch_bounds__(B::NT, 1)
-    rr_moment_pass2_kernel(float *__restrict__ f, const float *__restrict__ a,
-                           float *__restrict__ b, const Grid g, const float om1, const Pass2 p) {
+    rr_moment_pass2_kernel(float *f, const float *a, float *b, const Grid g, const float om1, const Pass2 p) {
   constexpr int K = B::K, NT = B::NT, SLOT = B::SLOT, P = K / 2;
   constexpr int kStride = B::STRIDE, kGuard = B::GUARD;
   extern __shared__ __align__(128) float sm[];
@@ -75,6 +75,7 @@ __global__ void __launch_bounds__(B::NT, 1)
     y = ya + ey;
     return c < cells;
   };
+  chain_wait();
 #pragma unroll
   for (int j = 0; j < K; ++j) {
     int x, y;
@@ -107,8 +108,8 @@ __global__ void __launch_bounds__(B::NT, 1)
       lane(mj.yy, k) = q.yy.x;
     } else {
       const float *src = a + block2(g, x, y);
-      const float4 u = __ldg(reinterpret_cast<const float4 *>(src) + (x & 31));
-      const float2 w = __ldg(reinterpret_cast<const float2 *>(src + 128) + (x & 31));
+      const float4 u = reinterpret_cast<const float4 *>(src)[x & 31];
+      const float2 w = reinterpret_cast<const float2 *>(src + 128)[x & 31];
       lane(mj.drho, k) = u.x;
       lane(mj.jx, k) = u.y;
       lane(mj.jy, k) = u.z;
@@ -224,8 +225,7 @@ cudaError_t pass2_t(float *f, const float *a, float *b, const Grid &g, float om1
   constexpr int smem = B::BUFS * 8 * B::SLOT * 4;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return e;
-  kern<<<blocks, B::NT, smem, st>>>(f, a, b, g, om1, p);
-  return cudaGetLastError();
+  return launch_chained(kern, blocks, B::NT, smem, st, f, a, b, g, om1, p);
 }
 template <int KIND>
 cudaError_t pass2_k(float *f, const float *a, float *b, const Grid &g, float om1, const Pass2 &p,

@@ -13,6 +13,7 @@
 // issue at half rate, 67% busy) and its dependent chains at 24 warps an SM;
 // with one cell a thread the same walk took 33.3 us (200 instructions a cell
 // instead of 139), with loads one row ahead instead of kAhead 45.6.
+#include "lbrr_chain.cuh"
 #include "lbrr_two.cuh"
 
 namespace lbrr {
@@ -45,8 +46,7 @@ struct PassM {
 // with one collision more.
 template <int EX, int KIND>
 __global__ void __launch_bounds__(kThreads2, 2)
-    rr_moment_march_kernel(float *__restrict__ f, const float *__restrict__ a,
-                           float *__restrict__ b, const Grid g, const float om1, const PassM p) {
+    rr_moment_march_kernel(float *f, const float *a, float *b, const Grid g, const float om1, const PassM p) {
   constexpr int H = EX / 2;
   constexpr int RS = EX + 4;      // a row of one population, with guard cells at its ends
   constexpr int BUF = 9 * RS;     // one row of all populations
@@ -101,6 +101,7 @@ __global__ void __launch_bounds__(kThreads2, 2)
     }
     asm volatile("cp.async.commit_group;" ::: "memory");
   };
+  chain_wait();
   if (u == 0)
     for (int k = 0; k < kAhead - 1; ++k) fetch();
 
@@ -223,8 +224,7 @@ cudaError_t passm_t(float *f, const float *a, float *b, const Grid &g, float om1
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
   }
-  kern<<<blocks, EX / 2 * (p.units + 1), smem, st>>>(f, a, b, g, om1, p);
-  return cudaGetLastError();
+  return launch_chained(kern, blocks, EX / 2 * (p.units + 1), smem, st, f, a, b, g, om1, p);
 }
 template <int KIND>
 cudaError_t passm_k(int ex, float *f, const float *a, float *b, const Grid &g, float om1,
