@@ -15,7 +15,10 @@
 // from a valid (unrelated) location before it is replaced.
 //
 // One thread per node, blocks along x; bytes per update as in the periodic
-// kernel. Any storage precision.
+// kernel. Any storage precision. Updates are chained (lbrr_chain.cuh): D3Q27 of
+// 64^3 nodes 11.1 -> 9.3 us an update, D2Q9 of 1001^2, whose store L2 delivers
+// at 7 TB/s, 10.25 -> 10.05.
+#include "lbrr_chain.cuh"
 #include "lbrr_launch.h"
 
 namespace lbrr {
@@ -46,6 +49,7 @@ __global__ void __launch_bounds__(kWallThreads)
   auto row = [&](int b, int c) -> long long { return ((long long)zs[c] * g.ny + ys[b]) * g.nx; };
   const long long cell = row(1, 1) + x;
 
+  chain_wait();
   if (PARITY == 0) {
 #pragma unroll
     for (int i = 0; i < Q; ++i) df[i] = St::template load<Q>(f + i * n + cell, i);
@@ -85,13 +89,8 @@ template <int Q, int S, int MODEL>
 static cudaError_t walls_t(void *f, const Grid &g, float om1, int parity, cudaStream_t st) {
   using T = typename Storage<S>::T;
   const dim3 grid((g.nx + kWallThreads - 1) / kWallThreads, g.ny, g.nz);
-  if (parity == 0)
-    rr_step_walls_kernel<Q, S, MODEL, 0><<<grid, kWallThreads, 0, st>>>(static_cast<T *>(f), g,
-                                                                         om1);
-  else
-    rr_step_walls_kernel<Q, S, MODEL, 1><<<grid, kWallThreads, 0, st>>>(static_cast<T *>(f), g,
-                                                                         om1);
-  return cudaGetLastError();
+  auto kern = parity ? rr_step_walls_kernel<Q, S, MODEL, 1> : rr_step_walls_kernel<Q, S, MODEL, 0>;
+  return launch_chained(kern, grid, kWallThreads, 0, st, static_cast<T *>(f), g, om1);
 }
 
 template <int Q, int S>
