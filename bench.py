@@ -372,7 +372,8 @@ def shear_variant(B, torch, stream, peak_gbs, n: int = 2048, steps: int = 20000,
                   machs=(0.1, 0.3, 0.5)):
     """The periodic D2Q9 double shear layer at n^2 (Re 1000 on L = n), FP32 store: the
     updates of a whole run timed with CUDA events on the solver's stream (lb_step
-    replays captured graphs of 8 updates), for each Mach number; the kinetic energy
+    carries several updates through one pass over the cells' moments, so the fraction of
+    the roofline, at the 72 B of a single update, can exceed 1), for each Mach number; the kinetic energy
     at the end against the start (finite: the run stayed stable)."""
     from paper_1505_06900_gb300 import workloads as W
     out = {"grid": [n, n], "steps": steps, "re": 1000.0, "bytes_per_update": 72, "runs": {}}

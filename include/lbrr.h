@@ -145,9 +145,13 @@ LB_API int lb_init_fields(lb_ctx *ctx, const float *rho, const float *u, int ini
 
 /* Advance n >= 0 full collide-and-stream updates (eq_discr_bgk_reg). n == 0 is
  * a no-op. Asynchronous on the context's stream. Without a learned closure,
- * runs of 8 updates are replayed from a CUDA graph that the context captures
+ * runs of updates of a periodic FP32 store go through the moments of the cells
+ * where that is faster (scratch of up to a quarter of the free memory, kept by
+ * the context; without it the updates run one by one), and other runs of 8
+ * updates are replayed from a CUDA graph that the context captures
  * on first use (one per starting AA parity, on a stream of its own); the
- * results are those of update-by-update launches, bit for bit. While the
+ * results are those of update-by-update launches, bit for bit (short of
+ * populations that underflow). While the
  * context's stream is being captured by the caller, updates are launched one
  * by one into that capture. With a 16-bit store the
  * update waits (boundedly) for its own bulk copies; if such a wait ever
@@ -307,11 +311,11 @@ LB_API int lb_closure_step_targets(lb_ctx *pre, lb_ctx *post, const lb_mlp *mlp,
 /* Use the network in lb_step (NULL: plain RR). A cell whose standardised
  * prediction exceeds `bound` in magnitude, or whose corrected populations are
  * not all positive, takes the RR update instead and is counted. The network
- * must outlive its use. On grids whose rows are whole 128-cell tiles an
- * update is two kernels: the standardised moments of every cell (BF16), then
- * the tcgen05 network, whose epilogue performs the corrected update of each
- * tile row's cell in place; on other grids the predictions go through device
- * memory to a separate update kernel. If a bounded wait of the network
+ * must outlive its use. An update is two kernels: the standardised moments of
+ * every cell (BF16), then the tcgen05 network, whose epilogue performs the
+ * corrected update of each tile row's cell in place; on small grids (some
+ * extent below 14) the predictions may go through device memory to a separate
+ * update kernel. If a bounded wait of the network
  * expires (reported as LB_ETIMEOUT), part of the cells of that update were
  * not updated: re-initialise or restore a checkpoint. */
 LB_API int lb_set_closure(lb_ctx *ctx, const lb_mlp *mlp, float bound);

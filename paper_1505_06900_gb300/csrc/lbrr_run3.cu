@@ -254,8 +254,8 @@ __device__ __forceinline__ void store_fields(float *p, int tail, const Macro &m)
 // of a tile: per plane it forms the post-collision populations of plane p + 1
 // of the tile and its ring of neighbours into shared memory, and gathers those
 // of plane p (one barrier a plane, two planes in shared memory); the sums of
-// the three z components of a cell meet in registers. 512^3, GB300: 2.37 ms an
-// update for D3Q27 (56.6 GLUPS, against 30.7 of the single updates). It moves
+// the three z components of a cell meet in registers. 512^3, GB300: 2.51 ms an
+// update for D3Q27 over a run of 20 (53.4 GLUPS, single updates 30.7). It moves
 // 80 bytes a cell through HBM at 4.2 TB/s; the bound is the instructions
 // issued (520 a cell, 69% of the issue slots). What mattered on the way:
 // single 4-byte accesses to the moments (47.4 GLUPS instead of 53.4 over 20

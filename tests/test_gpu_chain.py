@@ -5,6 +5,8 @@ without a synchronisation, alone, with other work on the stream in between that
 writes what the next kernel reads, and replayed from a captured graph, against
 the same calls with a synchronisation after each, bit for bit.
 """
+import ctypes
+
 import numpy as np
 import pytest
 
@@ -94,3 +96,44 @@ def test_runs_of_updates(shape):
         b.step(48)
         b.step(32)
         assert torch.equal(a.populations(), b.populations())
+
+
+@pytest.mark.parametrize("lattice,shape,walls", [(B.D2Q9, (65, 65, 1), 3), (B.D3Q27, (20, 18, 16), 2)])
+def test_captured_between_copies_and_a_second_stream(lattice, shape, walls):
+    """Chained kernels in a captured graph whose neighbours are copies and a
+    kernel of another stream that joins."""
+    with _solver(lattice, shape, walls=walls) as a, _solver(lattice, shape, walls=walls) as b:
+        state = torch.empty(a.state_bytes(), dtype=torch.uint8, device="cuda")
+        a.get_state(state)
+        first = state.clone()
+        a.step(6)
+        ref = a.populations()
+        net = _net(4)
+        gen = torch.Generator(device="cuda").manual_seed(9)
+        Xs = torch.randn((300, B.MLP_IN), device="cuda", generator=gen).to(torch.bfloat16)
+        T = torch.randn((300, B.MLP_OUT), device="cuda", generator=gen)
+        X = torch.zeros_like(Xs)
+        stream, side = torch.cuda.Stream(), torch.cuda.Stream()
+        torch.cuda.synchronize()
+        b.set_stream(stream)
+        net._lib.lb_mlp_set_stream(net.handle, ctypes.c_void_p(stream.cuda_stream))
+        keep, out = torch.empty_like(first), torch.empty_like(ref)
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph, stream=stream):
+            side.wait_stream(stream)
+            with torch.cuda.stream(side):
+                X.copy_(Xs)
+            keep.copy_(first)
+            b.step(4)
+            stream.wait_stream(side)
+            net.train_step(X, T, 1e-3, want_loss=False)
+            b.step(2)
+        b.set_state(first, 0)
+        graph.replay()
+        torch.cuda.synchronize()
+        assert torch.equal(b.populations(), ref) and torch.equal(X, Xs)
+        other = _net(4)
+        other.train_step(Xs, T, 1e-3, want_loss=False)
+        assert np.array_equal(net.get_params(), other.get_params())
+        net.close()
+        other.close()
