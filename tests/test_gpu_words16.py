@@ -13,6 +13,7 @@ import test_gpu_lowprec as T
 from paper_1505_06900_gb300 import binding as B
 
 pytestmark = pytest.mark.gpu
+torch = pytest.importorskip("torch")
 
 
 @pytest.mark.parametrize("storage", [B.STORE_F16, B.STORE_BF16])
@@ -26,3 +27,30 @@ pytestmark = pytest.mark.gpu
 ])
 def test_one_update(storage, parity, collision, lattice, shape):
     T.test_one_update_is_correctly_rounded(storage, parity, collision, lattice, shape)
+
+
+@pytest.mark.parametrize("storage", [B.STORE_F16, B.STORE_BF16])
+@pytest.mark.parametrize("lattice,shape,copies", [
+    (O.D2Q9, (250, 50, 1), 12), (O.D3Q19, (30, 20, 11), 10), (O.D3Q27, (26, 18, 10), 10),
+])
+def test_updates_equal_those_of_one_cell_to_a_thread(storage, lattice, shape, copies):
+    """A periodic pattern repeated along the last axis fills a store that takes
+    two cells to a thread, the pattern alone one that does not: populations bit
+    for bit over updates from both parities."""
+    _, q = O.dims_of(lattice)
+    axis = -2 if shape[2] == 1 else -3
+    long = (shape[0], shape[1] * copies, 1) if axis == -2 else shape[:2] + (shape[2] * copies,)
+    assert q * shape[0] * shape[1] * shape[2] < 1250000 <= q * long[0] * long[1] * long[2]
+    df = torch.from_numpy(T.W.random_populations(q, shape, seed=5, amp=0.05).astype("float32")).cuda()
+
+    def repeated(t):
+        return torch.cat([t] * copies, dim=axis)
+
+    with B.Solver(lattice, shape, 0.63, storage=storage) as a, \
+            B.Solver(lattice, long, 0.63, storage=storage) as b:
+        a.set_populations(df)
+        b.set_populations(repeated(df).contiguous())
+        for _ in range(3):
+            a.step(1)
+            b.step(1)
+            assert torch.equal(repeated(a.populations()), b.populations())
