@@ -848,6 +848,19 @@ int lb_mlp_train_step(lb_mlp *m, const void *X, const float *T, long long M, flo
   return mlp_backward(m, X, T, M, nullptr, 1, lr, loss);
 }
 
+// Zeros fresh device memory, done when the call returns: what follows on any
+// stream finds it so. (A memset on the legacy stream returns before it is done
+// and nothing orders it before the work of a non-blocking stream.)
+static cudaError_t zero_now(void *p, size_t bytes) {
+  cudaStream_t st = nullptr;
+  cudaError_t e = cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking);
+  if (e != cudaSuccess) return e;
+  e = cudaMemsetAsync(p, 0, bytes, st);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+  cudaStreamDestroy(st);
+  return e;
+}
+
 // Closure scratch: the moment field (lb_closure_features), and for the step
 // (for_step) the feature source of the TMA-fed network with its map, or, on
 // the grids that it does not take, the moment field and the predictions.
@@ -860,9 +873,9 @@ static int ensure_mom(lb_ctx *c, bool for_step) {
   if (e == cudaSuccess && conv && !c->xs) {
     e = cudaMalloc(&c->xs, lbrr::feature_source_bytes(c->g));
     if (e == cudaSuccess) {
-      // the row padding beyond the halo is copied by the last tile of a row
-      // but read by no MMA: zero it once
-      cudaError_t ez = cudaMemset(c->xs, 0, lbrr::feature_source_bytes(c->g));
+      // for the row padding beyond the halo, which no update writes: rows of whole
+      // tiles only copy it, other grids multiply it into tile rows that are dropped
+      cudaError_t ez = zero_now(c->xs, lbrr::feature_source_bytes(c->g));
       if (ez == cudaSuccess) ez = lbrr::make_feature_map(c->xs, c->g, &c->xs_map);
       if (ez != cudaSuccess) {
         cudaGetLastError();
@@ -891,9 +904,10 @@ int lb_closure_features(lb_ctx *c, const lb_mlp *m, void *X) {
   if (!m || !X) return fail(c, LB_EINVAL, "null argument");
   LB_NEED_DEVICE(c, X);
   int rc = closure_capable(c);
-  if (rc == LB_OK) rc = ensure_mom(c, false);
   if (rc != LB_OK) return rc;
   DeviceGuard dg(c->device);
+  rc = ensure_mom(c, false);
+  if (rc != LB_OK) return rc;
   cudaError_t e = lbrr::launch_moment_field(c->storage, c->f, c->g, c->parity, c->mom, c->stream);
   if (e == cudaSuccess) e = lbrr::launch_features(m->d, c->mom, c->g, X, c->stream);
   if (e != cudaSuccess) return cuda_fail(c, e, "closure features");
@@ -977,14 +991,17 @@ int lb_set_closure_ex(lb_ctx *c, const lb_mlp *m, float bound, float dead_zone) 
   if (!(dead_zone >= 0.f) || !std::isfinite(dead_zone))
     return fail(c, LB_EINVAL, "dead_zone must be a finite number >= 0");
   int rc = closure_capable(c);
-  if (rc == LB_OK) rc = ensure_mom(c, true);
   if (rc != LB_OK) return rc;
   DeviceGuard dg(c->device);
+  rc = ensure_mom(c, true);
+  if (rc != LB_OK) return rc;
   if (!c->fallbacks) {
     cudaError_t e = cudaMalloc(&c->fallbacks, sizeof(unsigned long long));
-    if (e == cudaSuccess) e = cudaMemset(c->fallbacks, 0, sizeof(unsigned long long));
+    if (e == cudaSuccess) e = zero_now(c->fallbacks, sizeof(unsigned long long));
     if (e != cudaSuccess) {
       cudaGetLastError();
+      cudaFree(c->fallbacks);
+      c->fallbacks = nullptr;
       return fail(c, LB_ENOMEM, "cannot allocate the fallback counter");
     }
   }
