@@ -27,7 +27,7 @@ constexpr int kWallThreads = 128;
 
 template <int Q, int S, int MODEL, int PARITY>
 __global__ void __launch_bounds__(kWallThreads)
-    rr_step_walls_kernel(typename Storage<S>::T *__restrict__ f, const Grid g, const float om1) {
+    rr_step_walls_kernel(typename Storage<S>::T *f, const Grid g, const float om1) {
   using St = Storage<S>;
   using L = Lattice<Q>;
   constexpr int D = L::D;
