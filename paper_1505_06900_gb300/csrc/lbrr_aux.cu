@@ -254,11 +254,13 @@ __global__ void __launch_bounds__(kRedThreads)
 // 0.5 |curl u|^2 per cell. FP64 arithmetic runs at a 64th of the FP32 rate on
 // this GPU and bounded this kernel (991 us for 256^3, whose field is read in
 // 40), so a component of the curl is formed as an unevaluated sum of two
-// floats by error-free transformations (Knuth's sum, an FMA for the square;
-// relative error below 2^-44), summed the same way over up to kCurlFlush cells,
-// and only that sum goes to FP64, between loops. A component whose square
-// would leave the range where its low part is an FP32 number, and the nodes on
-// walls, take FP64. With a cell to a thread that took 227 us, waiting for
+// floats by error-free transformations (Knuth's sum, an FMA for the square),
+// summed the same way over up to kCurlFlush cells, and only that sum goes to
+// FP64, between loops. The two differences of a component may cancel: its
+// rounding errors are kept until the leading terms have met, so it comes out to
+// 2^-47 of itself while these leave 2^-16 of their size. A component that
+// leaves less, or whose square would leave the range where its low part is an
+// FP32 number, and the nodes on walls, take FP64. With a cell to a thread that took 227 us, waiting for
 // twelve scalar loads; with four cells of a row, which the float4 rows of
 // nx % 4 == 0 allow, 106 us.
 constexpr int kCurlFlush = 64;
@@ -393,19 +395,25 @@ __global__ void __launch_bounds__(kRedThreads)
                            const float (&vm)[V]) {
 #pragma unroll
         for (int k = 0; k < V; ++k) {
-          float s1, e1, s2, e2, s, e;
+          float s1, e1, s2, e2, s, e, t, te;
           two_diff(up[k], um[k], s1, e1);
           two_diff(vp[k], vm[k], s2, e2);
           two_diff(s1, s2, s, e);
-          e += e1 - e2;
+          two_diff(e1, e2, t, te);
           const bool wall =
               plane || ((g.walls & 1) && ((k == 0 && x == 0) || (k == V - 1 && x + V == g.nx)));
           if (wall) continue;
           // NaN and infinities too
-          if (!(fabsf(s) >= 0x1p-45f && fabsf(s) <= 0x1p50f)) {
-            if (s != 0.f || e != 0.f) add_wide(&rare, up[k], um[k], vp[k], vm[k]);
+          const float size = fabsf(s);
+          if (!(size >= 0x1p-45f && size <= 0x1p50f &&
+                size >= 0x1p-16f * (fabsf(s1) + fabsf(s2)))) {
+            if (s != 0.f || t != 0.f) add_wide(&rare, up[k], um[k], vp[k], vm[k]);
             continue;
           }
+          e += t;  // s + e + te, and the first two with s leading
+          const float lead = s + e;
+          e = (e - (lead - s)) + te;
+          s = lead;
           const float q = s * s;
           part.add(q, fmaf(e, e, fmaf(2.0f * s, e, fmaf(s, s, -q))));
         }
