@@ -264,19 +264,25 @@ __global__ void __launch_bounds__(kRedThreads)
 // twelve scalar loads; with four cells of a row, which the float4 rows of
 // nx % 4 == 0 allow, 106 us.
 constexpr int kCurlFlush = 64;
+// The roundings that the transformations count on are asked for by name: a
+// product fused into the sum that follows would bring in its low part twice.
+__device__ __forceinline__ void two_sum(float a, float b, float &s, float &e) {
+  s = __fadd_rn(a, b);
+  const float v = __fsub_rn(s, a);
+  e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, v)), __fsub_rn(b, v));
+}
+__device__ __forceinline__ void two_diff(float a, float b, float &s, float &e) {
+  two_sum(a, -b, s, e);
+}
 struct Float2Sum {
   float s = 0.f, e = 0.f;
   __device__ __forceinline__ void add(float v, float err) {
-    const float t = s + v, b = t - s;
-    e += ((s - (t - b)) + (v - b)) + err;
+    float t, r;
+    two_sum(s, v, t, r);
+    e = __fadd_rn(e, __fadd_rn(r, err));
     s = t;
   }
 };
-__device__ __forceinline__ void two_diff(float a, float b, float &s, float &e) {
-  s = a - b;
-  const float v = s - a;
-  e = (a - (s - v)) - (b + v);
-}
 
 // FP64 work stays out of line and out of the loop's registers: as part of the
 // loop its operations were issued for every cell, predicated off (748 us).
@@ -410,12 +416,12 @@ __global__ void __launch_bounds__(kRedThreads)
             if (s != 0.f || t != 0.f) add_wide(&rare, up[k], um[k], vp[k], vm[k]);
             continue;
           }
-          e += t;  // s + e + te, and the first two with s leading
-          const float lead = s + e;
-          e = (e - (lead - s)) + te;
+          e = __fadd_rn(e, t);  // s + e + te, and the first two with s leading
+          const float lead = __fadd_rn(s, e);
+          e = __fadd_rn(__fsub_rn(e, __fsub_rn(lead, s)), te);
           s = lead;
-          const float q = s * s;
-          part.add(q, fmaf(e, e, fmaf(2.0f * s, e, fmaf(s, s, -q))));
+          const float q = __fmul_rn(s, s);
+          part.add(q, __fmaf_rn(e, e, __fmaf_rn(2.0f * s, e, __fmaf_rn(s, s, -q))));
         }
       };
       float up[V], um[V], vp[V], vm[V];
