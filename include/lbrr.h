@@ -150,8 +150,8 @@ LB_API int lb_init_fields(lb_ctx *ctx, const float *rho, const float *u, int ini
  * the context; without it the updates run one by one), and other runs of 8
  * updates are replayed from a CUDA graph that the context captures
  * on first use (one per starting AA parity, on a stream of its own); the
- * results are those of update-by-update launches, bit for bit (short of
- * populations that underflow). While the
+ * results are those of update-by-update launches, bit for bit (while the
+ * velocities are finite numbers). While the
  * context's stream is being captured by the caller, updates are launched one
  * by one into that capture. With a 16-bit store the
  * update waits (boundedly) for its own bulk copies; if such a wait ever

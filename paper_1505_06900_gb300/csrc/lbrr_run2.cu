@@ -11,16 +11,16 @@
 // take the kernel of lbrr_run2m.cu, which streams rows. The plan of a grid
 // (updates a pass, tiles, kernel) minimises an estimate fitted to both kernels.
 // Every value is computed by the operations of the single updates in their
-// order, so the store comes out bit for bit as theirs unless something
-// underflows. (Grids with walls stay with the single updates: the quiet
-// regions of a dipole do underflow, and the gain there was 5%, 10.1 -> 9.8 us
-// at 1001^2.)
+// order, so the store comes out bit for bit as theirs, underflow and the signs of
+// zeros included, while the velocities are finite numbers. (Grids with walls stay
+// with the single updates: the gain there was 5%, 10.1 -> 9.8 us at 1001^2.)
 //
-// GB300, microseconds an update, single updates / runs: 128^2 1.91 / 1.23 (50
-// updates), 251^2 2.14 / 1.90, 1001^2 9.57 / 8.12, 2048^2 46.2 / 28.0,
-// 4096x3000 134 / 75.7 (20 updates). The tile kernel issues in 39% of its
-// slots: its phases (collision, exchange, sums) follow one another in all warps
-// of a block, and one block fills an SM's registers.
+// GB300, microseconds an update, single updates / runs: 128^2 1.91 / 1.07 (50
+// updates), 251^2 2.14 / 1.69, 1001^2 9.57 / 7.50, 2048^2 46.2 / 28.2,
+// 4096x3000 134 / 75.8 (20 updates). The tile kernel issues in 39% (128^2) and
+// 45% (1001^2) of the slots of its active SMs: its phases (collision, exchange,
+// sums) follow one another in all warps of a block, and one block fills an SM's
+// registers.
 #include "lbrr_chain.cuh"
 #include "lbrr_two.cuh"
 
@@ -58,7 +58,8 @@ struct Pass2 {
 // collision more.
 template <class B, int KIND>
 __global__ void __launch_bounds__(B::NT, 1)
-    rr_moment_pass2_kernel(float *f, const float *a, float *b, const Grid g, const float om1, const Pass2 p) {
+    rr_moment_pass2_kernel(float *f, const float *a, float *b, const Grid g, const float om1,
+                           const Pass2 p) {
   constexpr int K = B::K, NT = B::NT, SLOT = B::SLOT, P = K / 2;
   constexpr int kStride = B::STRIDE, kGuard = B::GUARD;
   extern __shared__ __align__(128) float sm[];
@@ -98,7 +99,7 @@ __global__ void __launch_bounds__(B::NT, 1)
       load_logical<9, 0>(f, g, p.parity, x, y, 0, df);
       V v[9];
 #pragma unroll
-      for (int i = 0; i < 9; ++i) v[i] = bc(scale2(i) * df[i]);
+      for (int i = 0; i < 9; ++i) v[i] = bc(df[i]);
       Mom2 q = moments_of(v);
       lane(mj.drho, k) = q.drho.x;
       lane(mj.jx, k) = q.jx.x;
@@ -131,7 +132,8 @@ __global__ void __launch_bounds__(B::NT, 1)
         if (t + (2 * j + k) * NT < cells) {
 #pragma unroll
           for (int i = 0; i < 9; ++i)
-            if (i != 4) buf[(i < 4 ? i : i - 1) * SLOT + (k ? e[j] >> 16 : e[j] & 0xFFFFu)] = lane(q[i], k);
+            if (i != 4)
+              buf[(i < 4 ? i : i - 1) * SLOT + (k ? e[j] >> 16 : e[j] & 0xFFFFu)] = lane(q[i], k);
         }
       own[j] = q[4];
     }
@@ -163,7 +165,7 @@ __global__ void __launch_bounds__(B::NT, 1)
       if (KIND == 2) {
 #pragma unroll
         for (int i = 0; i < 9; ++i) {
-          const float v = lane(q[i], k) * (1.0f / scale2(i));
+          const float v = lane(q[i], k);
           if (p.parity == 1)
             f[(8 - i) * n + (long long)y * g.nx + x] = v;
           else
@@ -239,9 +241,9 @@ cudaError_t pass2_k(float *f, const float *a, float *b, const Grid &g, float om1
 }  // namespace
 
 // Fewer than six updates do not pay for the first and last passes, which touch
-// the store (1001^2: 12.3 us an update singly, 15.4 as a run of 4, 10.1 as one
+// the store (1001^2: 12.3 us an update singly, 15.4 as a run of 4, 9.8 as one
 // of 6), except on small grids, where launches count (128^2, 4 updates: 4.2 /
-// 3.8).
+// 3.2).
 bool moment_run2_supported(int q, int storage, int model, const Grid &g, int steps) {
   if (q != 9 || storage != 0 || model != 0 || g.walls) return false;
   return steps >= 6 || (steps >= 4 && g.n <= (1 << 19));

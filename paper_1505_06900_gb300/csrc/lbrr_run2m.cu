@@ -8,9 +8,11 @@
 // ends of a segment; memory is read and written once a pass, 48 bytes a cell
 // for three to eight updates. A thread has two cells, half a row apart, in
 // packed arithmetic: accesses stay coalesced and free of bank conflicts.
-// 2048^2, 50 updates: 28.0 us an update (150 GLUPS) against 46.2 of the single
+// 2048^2, 50 updates: 28.2 us an update (149 GLUPS) against 46.2 of the single
 // updates at 0.96 of the copy rate. Bound: the FMA pipe (packed operations
-// issue at half rate, 67% busy) and its dependent chains at 24 warps an SM;
+// issue at half rate; 53% busy over a pass that starts cold, and the warps wait
+// for it, for the row's barrier and for their dependent chains in about equal
+// parts) at 24 warps an SM;
 // with one cell a thread the same walk took 33.3 us (200 instructions a cell
 // instead of 139), with loads one row ahead instead of kAhead 45.6.
 #include "lbrr_chain.cuh"
@@ -46,7 +48,8 @@ struct PassM {
 // with one collision more.
 template <int EX, int KIND>
 __global__ void __launch_bounds__(kThreads2, 2)
-    rr_moment_march_kernel(float *f, const float *a, float *b, const Grid g, const float om1, const PassM p) {
+    rr_moment_march_kernel(float *f, const float *a, float *b, const Grid g, const float om1,
+                           const PassM p) {
   constexpr int H = EX / 2;
   constexpr int RS = EX + 4;      // a row of one population, with guard cells at its ends
   constexpr int BUF = 9 * RS;     // one row of all populations
@@ -116,7 +119,7 @@ __global__ void __launch_bounds__(kThreads2, 2)
         V df[9];
 #pragma unroll
         for (int i = 0; i < 9; ++i)
-          df[i] = muls(scale2(i), make_float2(from[i * EX + ex], from[i * EX + ex + H]));
+          df[i] = make_float2(from[i * EX + ex], from[i * EX + ex + H]);
         m = moments_of(df);
       } else {
         const float4 *q4 = reinterpret_cast<const float4 *>(from) + ex;
@@ -161,7 +164,7 @@ __global__ void __launch_bounds__(kThreads2, 2)
           if (out[c] && y >= y0 && y < y1) {
 #pragma unroll
             for (int i = 0; i < 9; ++i) {
-              const float v = lane(q[i], c) * (1.0f / scale2(i));
+              const float v = lane(q[i], c);
               if (p.parity == 1)
                 f[(8 - i) * n + (long long)y * g.nx + xu[c]] = v;
               else

@@ -1,31 +1,36 @@
 // Runs of updates of a periodic 3-D FP32 grid carried out on its moments.
 //
 // The regularized collision (RR and its order-2 form) replaces the
-// populations of a cell by a function of ten numbers: rho - 1, rho u and
-// Pi^(1) (Sec. 3.5). So between the first and the last of a run of updates
-// the state need not be kept as Q populations: an update reads the ten moments
-// of every cell, forms the post-collision populations, streams them inside
-// the chip and reduces them to the ten moments of the next state, 80 bytes
-// a cell instead of 2 Q 4 (216 for D3Q27). The run starts with the moments of
-// the AA store and ends with its last collision streamed into the store, in
-// the layout the same number of single updates would leave. Every value is
-// computed by the operations of the single updates in their order (the
-// moments' sums over x, y, then z are split by z component), so the result is
-// theirs bit for bit unless something underflows.
+// populations of a cell by a function of ten numbers: rho - 1, rho u and the
+// second moments, from which Pi^(1) follows (Sec. 3.5). So between the first and
+// the last of a run of updates the state need not be kept as Q populations: an
+// update reads the ten moments of every cell, forms the post-collision
+// populations, streams them inside the chip and reduces them to the ten moments
+// of the next state, 80 bytes a cell instead of 2 Q 4 (216 for D3Q27). The run
+// starts with the moments of the AA store and ends with its last collision
+// streamed into the store, in the layout the same number of single updates would
+// leave. Every value is computed by the operations of the single updates in
+// their order (the moments' sums over x, y, then z are split by z component), so
+// the result is theirs bit for bit, underflow and the signs of zeros included,
+// while the velocities are finite numbers.
 #include "lbrr_launch.h"
+#include "lbrr_quot.cuh"
 
 namespace lbrr {
 
 namespace {
 
-constexpr int kFields = 10;  // rho - 1, rho u (3), Pi^(1) (xx, xy, xz, yy, yz, zz)
+constexpr int kFields = 10;  // rho - 1, rho u (3), second moments (xx, xy, xz, yy, yz, zz)
 constexpr int kTX = 32, kEX = kTX + 2;  // cells of a tile row, with its neighbours
 
 // Tile of a block, one block per SM: as many threads as the registers allow
 // without spills (80 and 72 a thread: 24 and 28 warps), since the ring of
 // recomputed cells around the tile shrinks with its size. Measured at 256^3
 // (D3Q27 / D3Q19, GLUPS over 20 updates): 16 rows 47.1 / 55.3, 20 rows 49.0 /
-// 58.6, 24 rows 44.7 (72 registers) / 61.4, two blocks of 9 rows 46.8 / 57.3.
+// 58.6, 24 rows 44.7 (72 registers) / 61.4, two blocks of 9 rows 46.8 / 57.3 (all
+// with the populations of D3Q27 at twice their value or more inside the chip,
+// which saved factors of 1/2 but rounded what underflows differently; 47.7 / 60.8
+// as it is).
 template <int Q>
 struct Tile {
   static constexpr int TY = Q == 27 ? 20 : 24, EY = TY + 2, E = kEX * EY;
@@ -68,69 +73,23 @@ constexpr int plane_shared() {  // floats of one plane in shared memory
   return (2 * outers<Q>() + 8) * Tile<Q>::E;
 }
 
-// The chip-internal form of the D3Q27 populations: population i times
-// 2^(number of its non-zero velocity components). The 1-D synthesis is then
-// (q - c1, c0 - q, q + c1) with q = c2 + c0 / 3, without its factors 1/2, and
-// the sums below put them back; powers of two change no rounding.
-__device__ __forceinline__ void synth1x(float c0, float c1, float c2, float &om, float &oz,
-                                        float &op) {
-  const float q = fmaf(c0, kCs2, c2);
-  oz = c0 - q;
-  op = q + c1;
-  om = q - c1;
-}
-template <int MODEL>
-__device__ __forceinline__ void post_collision(const Macro &m, float om1, float (&f)[27]) {
-  float c[3][3][3], sx[3][3][3], sy[3][3][3];
-  if (MODEL == 0)
-    coeffs_rr_d3q27(m, om1, c);
-  else
-    coeffs_reg2_d3q27(m, om1, c);
-#pragma unroll
-  for (int j = 0; j < 9; ++j)
-    synth1x(c[0][j / 3][j % 3], c[1][j / 3][j % 3], c[2][j / 3][j % 3], sx[0][j / 3][j % 3],
-            sx[1][j / 3][j % 3], sx[2][j / 3][j % 3]);
-#pragma unroll
-  for (int j = 0; j < 9; ++j)
-    synth1x(sx[j / 3][0][j % 3], sx[j / 3][1][j % 3], sx[j / 3][2][j % 3], sy[j / 3][0][j % 3],
-            sy[j / 3][1][j % 3], sy[j / 3][2][j % 3]);
-#pragma unroll
-  for (int j = 0; j < 9; ++j)  // j = ix + 3 iy
-    synth1x(sy[j % 3][j / 3][0], sy[j % 3][j / 3][1], sy[j % 3][j / 3][2], f[j], f[j + 9],
-            f[j + 18]);
-}
-template <int MODEL>
-__device__ __forceinline__ void post_collision(const Macro &m, float om1, float (&f)[19]) {
-  Lattice<19>::template synth<MODEL>(m, om1, f);
-}
-
 // The sums of one z component: x lines, then y (sum, first and second moments
-// of total order <= 2), as moments_d3q27 and moments_d3q19 form them. On the
-// scaled D3Q27 populations x, y, xx, yy come out doubled and xy fourfold, and
-// all six once more doubled for z components -1 and +1.
-template <bool SCALED>
-__device__ __forceinline__ void sum3(float a, float b, float c, float &s0, float &s1, float &s2) {
-  s2 = a + c;
-  s0 = SCALED ? fmaf(0.5f, s2, b) : s2 + b;
-  s1 = c - a;
-}
+// of total order <= 2), as moments_d3q27 and moments_d3q19 form them.
 struct Part {
   float s, x, y, xx, yy, xy;
 };
-template <bool SCALED>
 __device__ __forceinline__ Part part(const float (&f)[9]) {
   float x0[3], x1[3], x2[3], t0, t1, t2;
 #pragma unroll
   for (int l = 0; l < 3; ++l)
-    sum3<SCALED>(f[3 * l], f[3 * l + 1], f[3 * l + 2], x0[l], x1[l], x2[l]);
+    mom3<false>(f[3 * l], f[3 * l + 1], f[3 * l + 2], x0[l], x1[l], x2[l]);
   Part p;
-  sum3<SCALED>(x0[0], x0[1], x0[2], p.s, p.y, p.yy);
-  sum3<SCALED>(x1[0], x1[1], x1[2], p.x, p.xy, t0);
-  sum3<SCALED>(x2[0], x2[1], x2[2], p.xx, t1, t2);
+  mom3<false>(x0[0], x0[1], x0[2], p.s, p.y, p.yy);
+  mom3<false>(x1[0], x1[1], x1[2], p.x, p.xy, t0);
+  mom3<false>(x2[0], x2[1], x2[2], p.xx, t1, t2);
   return p;
 }
 // the cross (0,-1), (-1,0), (0,0), (1,0), (0,1) of a D3Q19 plane z = +-1
-template <bool>
 __device__ __forceinline__ Part part(const float (&f)[5]) {
   Part p;
   p.xx = f[1] + f[3];
@@ -141,85 +100,73 @@ __device__ __forceinline__ Part part(const float (&f)[5]) {
   p.xy = 0.0f;
   return p;
 }
-// a / b correctly rounded, from r = the correctly rounded 1 / b: one correction
-// of the quotient by its exact remainder (P. Markstein, IBM J. Res. Dev. 34,
-// 1990). One reciprocal serves the three components of a velocity.
-__device__ __forceinline__ float quot(float a, float b, float r) {
-  const float q = __fmul_rn(a, r);
-  return __fmaf_rn(__fmaf_rn(-b, q, a), r, q);
-}
-__device__ __forceinline__ void set_velocity(Macro &m) {
-  const float r = __frcp_rn(m.rho);
-  m.ux = quot(m.jx, m.rho, r);
-  m.uy = quot(m.jy, m.rho, r);
-  m.uz = quot(m.jz, m.rho, r);
-}
+// What a cell carries from update to update: rho - 1, rho u and its raw second
+// moments.
+struct Mom3 {
+  float drho, jx, jy, jz, xx, xy, xz, yy, yz, zz;
+};
 
-// Macroscopic values from raw moments, as macro_from_moments. A single update
-// rounds a product j_a u_b before it takes it from the second moment where
-// its synthesis uses the product too (order-2 form: all; D3Q19: the diagonal
-// ones); elsewhere the difference is one fused operation.
+// a / b correctly rounded, from nr = minus the correctly rounded 1 / b: one
+// correction of the quotient by its exact remainder (P. Markstein, IBM J. Res.
+// Dev. 34, 1990; taken so that a zero keeps its sign). One reciprocal serves the
+// three components of a velocity.
+__device__ __forceinline__ float quot(float a, float b, float nr) {
+  const float q = __fmul_rn(-a, nr);
+  return __fmaf_rn(__fmaf_rn(b, q, -a), nr, q);
+}
+// Macroscopic values as macro_from_moments forms them. A single update rounds a
+// product j_a u_b before it takes it from the second moment where its synthesis
+// uses the product too (order-2 form: all; D3Q19: the diagonal ones); elsewhere
+// the difference is one fused operation.
 template <int Q, int MODEL>
-__device__ __forceinline__ Macro macro_raw(float m0, float jx, float jy, float jz, float pxx,
-                                           float pyy, float pzz, float pxy, float pxz,
-                                           float pyz) {
+__device__ __forceinline__ Macro macro_of(const Mom3 &v) {
   Macro m;
-  m.drho = m0;
-  m.rho = 1.0f + m0;
-  m.jx = jx;
-  m.jy = jy;
-  m.jz = jz;
-  set_velocity(m);
+  m.drho = v.drho;
+  m.rho = 1.0f + v.drho;
+  m.jx = v.jx;
+  m.jy = v.jy;
+  m.jz = v.jz;
+  const float nr = minus_reciprocal(m.rho);
+  m.ux = quot(m.jx, m.rho, nr);
+  m.uy = quot(m.jy, m.rho, nr);
+  m.uz = quot(m.jz, m.rho, nr);
+  if (!(fminf(fminf(fabsf(m.ux), fabsf(m.uy)), fabsf(m.uz)) >= kLeastQuotient)) {
+    if (needs_division(m.jx, m.ux) || needs_division(m.jy, m.uy) || needs_division(m.jz, m.uz)) {
+      m.ux = __fdiv_rn(m.jx, m.rho);
+      m.uy = __fdiv_rn(m.jy, m.rho);
+      m.uz = __fdiv_rn(m.jz, m.rho);
+    }
+  }
   auto less = [](bool round, float p, float j, float u) {
     return round ? __fsub_rn(p, __fmul_rn(j, u)) : __fmaf_rn(-j, u, p);
   };
   constexpr bool off = Q == 27 && MODEL == 1, diag = off || Q == 19;
-  m.pxx = less(diag, __fmaf_rn(-kCs2, m0, pxx), jx, m.ux);
-  m.pyy = less(diag, __fmaf_rn(-kCs2, m0, pyy), jy, m.uy);
-  m.pzz = less(diag, __fmaf_rn(-kCs2, m0, pzz), jz, m.uz);
-  m.pxy = less(off, pxy, jx, m.uy);
-  m.pxz = less(off, pxz, jx, m.uz);
-  m.pyz = less(off, pyz, jy, m.uz);
+  m.pxx = less(diag, __fmaf_rn(-kCs2, m.drho, v.xx), m.jx, m.ux);
+  m.pyy = less(diag, __fmaf_rn(-kCs2, m.drho, v.yy), m.jy, m.uy);
+  m.pzz = less(diag, __fmaf_rn(-kCs2, m.drho, v.zz), m.jz, m.uz);
+  m.pxy = less(off, v.xy, m.jx, m.uy);
+  m.pxz = less(off, v.xz, m.jx, m.uz);
+  m.pyz = less(off, v.yz, m.jy, m.uz);
   return m;
 }
 
-// Macroscopic values from the sums of z component -1 (m), 0 (z) and +1 (p).
-template <int Q, int MODEL, bool SCALED>
-__device__ __forceinline__ Macro combine(const Part &m, const Part &z, const Part &p) {
-  constexpr float h = SCALED ? 0.5f : 1.0f, q = SCALED ? 0.25f : 1.0f;
-  auto sum = [](float a, float b, float c) { return SCALED ? fmaf(0.5f, a + c, b) : (a + c) + b; };
-  return macro_raw<Q, MODEL>(sum(m.s, z.s, p.s), h * sum(m.x, z.x, p.x), h * sum(m.y, z.y, p.y),
-                             h * (p.s - m.s), h * sum(m.xx, z.xx, p.xx),
-                             h * sum(m.yy, z.yy, p.yy), h * (m.s + p.s),
-                             Q == 27 ? q * sum(m.xy, z.xy, p.xy) : z.xy, q * (p.x - m.x),
-                             q * (p.y - m.y));
+// Moments from the sums of z component -1 (m), 0 (z) and +1 (p).
+template <int Q>
+__device__ __forceinline__ Mom3 combine(const Part &m, const Part &z, const Part &p) {
+  auto sum = [](float a, float b, float c) { return (a + c) + b; };
+  return {sum(m.s, z.s, p.s), sum(m.x, z.x, p.x), sum(m.y, z.y, p.y), p.s - m.s,
+          sum(m.xx, z.xx, p.xx), Q == 27 ? sum(m.xy, z.xy, p.xy) : z.xy, p.x - m.x,
+          sum(m.yy, z.yy, p.yy), p.y - m.y, m.s + p.s};
 }
-template <int Q, int MODEL>
-__device__ __forceinline__ Macro moments_of(const float (&f)[Q]) {
+template <int Q>
+__device__ __forceinline__ Mom3 moments_of(const float (&f)[Q]) {
   float gm[group_size<Q>(-1)], gz[group_size<Q>(0)], gp[group_size<Q>(1)];
 #pragma unroll
   for (int i = 0; i < Q; ++i) {
     constexpr int o = group_size<Q>(-1), w = o + group_size<Q>(0);
     (i < o ? gm[i] : (i < w ? gz[i - o] : gp[i - w])) = f[i];
   }
-  return combine<Q, MODEL, false>(part<false>(gm), part<false>(gz), part<false>(gp));
-}
-
-__device__ __forceinline__ Macro macro_of(const float (&v)[kFields]) {
-  Macro m;
-  m.drho = v[0];
-  m.rho = 1.0f + m.drho;
-  m.jx = v[1];
-  m.jy = v[2];
-  m.jz = v[3];
-  m.pxx = v[4];
-  m.pxy = v[5];
-  m.pxz = v[6];
-  m.pyy = v[7];
-  m.pyz = v[8];
-  m.pzz = v[9];
-  set_velocity(m);
-  return m;
+  return combine<Q>(part(gm), part(gz), part(gp));
 }
 
 // Layout of the moments: rows in blocks of 32 cells; of a block first the
@@ -236,30 +183,29 @@ __device__ __forceinline__ uint32_t cell_float(const Grid &g, int x, int y) {
 }
 // the two float2 fields of a cell, from its float4 address and x
 __device__ __forceinline__ int tail_float(int x) { return 256 - 2 * (x & 31); }
-__device__ __forceinline__ void load_fields(const float *p, int tail, float (&v)[kFields]) {
+__device__ __forceinline__ Mom3 load_fields(const float *p, int tail) {
   const float4 u = __ldg(reinterpret_cast<const float4 *>(p));
   const float4 w = __ldg(reinterpret_cast<const float4 *>(p + 128));
   const float2 r = __ldg(reinterpret_cast<const float2 *>(p + tail));
-  v[0] = u.x, v[1] = u.y, v[2] = u.z, v[3] = u.w;
-  v[4] = w.x, v[5] = w.y, v[6] = w.z, v[7] = w.w;
-  v[8] = r.x, v[9] = r.y;
+  return {u.x, u.y, u.z, u.w, w.x, w.y, w.z, w.w, r.x, r.y};
 }
-__device__ __forceinline__ void store_fields(float *p, int tail, const Macro &m) {
+__device__ __forceinline__ void store_fields(float *p, int tail, const Mom3 &m) {
   *reinterpret_cast<float4 *>(p) = make_float4(m.drho, m.jx, m.jy, m.jz);
-  *reinterpret_cast<float4 *>(p + 128) = make_float4(m.pxx, m.pxy, m.pxz, m.pyy);
-  *reinterpret_cast<float2 *>(p + tail) = make_float2(m.pyz, m.pzz);
+  *reinterpret_cast<float4 *>(p + 128) = make_float4(m.xx, m.xy, m.xz, m.yy);
+  *reinterpret_cast<float2 *>(p + tail) = make_float2(m.yz, m.zz);
 }
 
 // One update of the moments a -> b. A block walks the planes of a z segment
 // of a tile: per plane it forms the post-collision populations of plane p + 1
 // of the tile and its ring of neighbours into shared memory, and gathers those
 // of plane p (one barrier a plane, two planes in shared memory); the sums of
-// the three z components of a cell meet in registers. 512^3, GB300: 2.51 ms an
-// update for D3Q27 over a run of 20 (53.4 GLUPS, single updates 30.7). It moves
-// 80 bytes a cell through HBM at 4.2 TB/s; the bound is the instructions
-// issued (520 a cell, 69% of the issue slots). What mattered on the way:
-// single 4-byte accesses to the moments (47.4 GLUPS instead of 53.4 over 20
-// updates), 4-byte shared-memory accesses only and columns (0, 0) exchanged
+// the three z components of a cell meet in registers. 512^3, GB300: 2.59 ms an
+// update for D3Q27 over a run of 20 (51.7 GLUPS, single updates 30.7). It moves
+// 80 bytes a cell through HBM at 4.0 TB/s; the bound is the instructions
+// issued (547 a cell, 74% of the issue slots of the active SMs, three ready
+// warps waiting for every one that issues). What mattered on the way:
+// single 4-byte accesses to the moments (47.4 GLUPS where 53.4 were reached over
+// 20 updates), 4-byte shared-memory accesses only and columns (0, 0) exchanged
 // too (41.8), and any spill, since shared memory leaves the L1 cache little.
 template <int Q, int MODEL>
 __global__ void __launch_bounds__(Tile<Q>::kThreads, 1)
@@ -289,15 +235,15 @@ __global__ void __launch_bounds__(Tile<Q>::kThreads, 1)
   const int tail = tail_float(x);
   const int e = ey * kEX + ex;
 
-  float mv[kFields];
+  Mom3 mv;
   float own[3], next[3];  // the populations of velocity (0, 0, *), which stay in their column
   auto fetch = [&](int p) {
     const int zp = p < 0 ? p + g.nz : (p >= g.nz ? p - g.nz : p);
-    load_fields(a + zp * plane + cell, tail, mv);
+    mv = load_fields(a + zp * plane + cell, tail);
   };
   auto post = [&](int p) {
     float df[Q];
-    post_collision<MODEL>(macro_of(mv), om1, df);
+    Lattice<Q>::template synth<MODEL>(macro_of<Q, MODEL>(mv), om1, df);
     float *dst = sm + (p & 1) * plane_shared<Q>();
 #pragma unroll
     for (int c = 0; c < 9; ++c) {
@@ -342,11 +288,11 @@ __global__ void __launch_bounds__(Tile<Q>::kThreads, 1)
       }
       if (p > z0 && in) {
         store_fields(b + (p - 1) * plane + cell, tail,
-                     combine<Q, MODEL, Q == 27>(part<Q == 27>(gm), d1, c2));
+                     combine<Q>(part(gm), d1, c2));
       }
       c2 = c1;
-      c1 = part<Q == 27>(gp);
-      d1 = part<Q == 27>(gz);
+      c1 = part(gp);
+      d1 = part(gz);
     }
 #pragma unroll
     for (int k = 0; k < 3; ++k) own[k] = next[k];
@@ -357,7 +303,7 @@ __global__ void __launch_bounds__(Tile<Q>::kThreads, 1)
 constexpr int kCellThreads = 128;
 
 // Moments of the logical populations of an AA store of either parity.
-template <int Q, int MODEL>
+template <int Q>
 __global__ void __launch_bounds__(kCellThreads)
     moments_of_store_kernel(const float *__restrict__ f, const Grid g, const int parity,
                             float *__restrict__ b) {
@@ -366,7 +312,7 @@ __global__ void __launch_bounds__(kCellThreads)
   float df[Q];
   load_logical<Q, 0>(f, g, parity, x, blockIdx.y, blockIdx.z, df);
   store_fields(b + blockIdx.z * plane_floats(g) + cell_float(g, x, blockIdx.y), tail_float(x),
-               moments_of<Q, MODEL>(df));
+               moments_of<Q>(df));
 }
 
 // The update that ends a run: collision from the moments into the AA store, at
@@ -380,9 +326,9 @@ __global__ void __launch_bounds__(kCellThreads)
   if (x >= g.nx) return;
   const int y = blockIdx.y, z = blockIdx.z;
   const long long cell = ((long long)z * g.ny + y) * g.nx + x;
-  float v[kFields], df[Q];
-  load_fields(a + z * plane_floats(g) + cell_float(g, x, y), tail_float(x), v);
-  Lattice<Q>::template synth<MODEL>(macro_of(v), om1, df);
+  float df[Q];
+  const Mom3 v = load_fields(a + z * plane_floats(g) + cell_float(g, x, y), tail_float(x));
+  Lattice<Q>::template synth<MODEL>(macro_of<Q, MODEL>(v), om1, df);
 #pragma unroll
   for (int i = 0; i < Q; ++i) {
     if (PARITY == 1) {
@@ -429,7 +375,7 @@ cudaError_t run_t(float *f, float *m0, float *m1, const Grid &g, float om1, int 
   if (e != cudaSuccess) return e;
   const RunPlan r = plan_of(Tile<Q>::TY, g, sms);
   const dim3 cells((g.nx + kCellThreads - 1) / kCellThreads, g.ny, g.nz);
-  moments_of_store_kernel<Q, MODEL><<<cells, kCellThreads, 0, st>>>(f, g, parity, m0);
+  moments_of_store_kernel<Q><<<cells, kCellThreads, 0, st>>>(f, g, parity, m0);
   for (int k = 1; k < steps; ++k) {
     kern<<<r.blocks, threads, smem, st>>>(m0, m1, g, om1, r.tiles_x, r.tiles_y, r.seg);
     float *s = m0;
@@ -450,12 +396,12 @@ cudaError_t run_t(float *f, float *m0, float *m1, const Grid &g, float om1, int 
 // D3Q27, and the pass over the moments does not), and enough updates on a
 // grid its tiles fill. In units of a single update of every cell (216 or 152
 // bytes a cell at the copy rate), its first and last passes cost 296 / 216 or
-// 232 / 152, and an update between them 0.52 (D3Q27) or 0.60 (D3Q19) of the
+// 232 / 152, and an update between them 0.54 (D3Q27) or 0.60 (D3Q19) of the
 // cells its plane iterations could hold, which is what the kernel measures at
-// 256^3 and 512^3; 0.10 and 0.14 are added on the safe side. Measured on both
+// 256^3 and 512^3; 0.08 and 0.14 are added on the safe side. Measured on both
 // sides of the lines (microseconds an update, single / moments): 96x60x64
-// 10.5 / 15.3, 640x130x9 19.3 / 24.3, 128^3 70.3 / 51.4 (40 updates) and 72.7 /
-// 68.3 (3), 250x151x101 131 / 94.8; D3Q19 128^3 50.8 / 52.0 (6 updates),
+// 10.5 / 15.3, 640x130x9 19.3 / 24.3, 128^3 70.3 / 54.8 (40 updates) and 72.7 /
+// 69.3 (3), 250x151x101 131 / 97.2; D3Q19 128^3 50.8 / 52.0 (6 updates),
 // 160x145x130 73.8 / 70.9 (9).
 bool moment_run_supported(int q, int storage, int model, const Grid &g, int steps, int sms) {
   if (q == 9 || model == 2 || storage != 0 || g.walls || steps < 3 ||

@@ -4,6 +4,7 @@
 #pragma once
 
 #include "lbrr_launch.h"
+#include "lbrr_quot.cuh"
 
 namespace lbrr {
 namespace two {
@@ -11,7 +12,9 @@ namespace two {
 // ------------------------------------------------------ two cells at a time --
 // The collision of lbrr_device.cuh (RR on D2Q9) on float2 values, one packed
 // FP32x2 instruction of the sm_100 family an operation: the operations of the
-// single updates in their order, so the bits are theirs.
+// single updates in their order, so the bits are theirs. (With the outer
+// populations at twice their value inside the chip, which leaves factors of 1/2
+// out, a value that underflows was rounded elsewhere; 3% faster.)
 using V = float2;
 __device__ __forceinline__ V bc(float s) { return make_float2(s, s); }
 __device__ __forceinline__ V add(V a, V b) { return __fadd2_rn(a, b); }
@@ -30,66 +33,68 @@ struct Mac2 {
   V drho, rho, jx, jy, ux, uy, pxx, pxy, pyy;
 };
 
-// j / rho correctly rounded (P. Markstein, IBM J. Res. Dev. 34, 1990): one
-// Newton step takes the 1-ulp approximation to the correctly rounded
-// reciprocal, one correction by the exact remainder the quotient to its own.
-__device__ __forceinline__ float rcp_approx(float x) {
-  float r;
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
-  return r;
+// minus_reciprocal of both
+__device__ __forceinline__ V minus_reciprocals(V x) {
+  const V r = make_float2(approx_reciprocal(-x.x), approx_reciprocal(-x.y));
+  return fma(fma(x, r, bc(1.0f)), r, r);
 }
-__device__ __forceinline__ void set_velocity(Mac2 &m) {
-  m.rho = add(bc(1.0f), m.drho);
-  const V nr = muls(-1.0f, m.rho);
-  V r = make_float2(rcp_approx(m.rho.x), rcp_approx(m.rho.y));
-  r = fma(fma(nr, r, bc(1.0f)), r, r);
-  const V qx = mul(m.jx, r), qy = mul(m.jy, r);
-  m.ux = fma(fma(nr, qx, m.jx), r, qx);
-  m.uy = fma(fma(nr, qy, m.jy), r, qy);
-}
+// u = j / rho correctly rounded: the quotient by the reciprocal of rho, corrected
+// by its exact remainder (P. Markstein, IBM J. Res. Dev. 34, 1990; taken as
+// rho q - j, with minus the reciprocal, so that a zero keeps its sign).
 __device__ __forceinline__ Mac2 macro_of(const Mom2 &v) {
   Mac2 m;
   m.drho = v.drho;
+  m.rho = add(bc(1.0f), m.drho);
   m.jx = v.jx;
   m.jy = v.jy;
-  set_velocity(m);
-  const V nx = muls(-1.0f, m.jx);
+  const V nx = muls(-1.0f, m.jx), ny = muls(-1.0f, m.jy);
+  const V nr = minus_reciprocals(m.rho);
+  const V qx = mul(nx, nr), qy = mul(ny, nr);
+  m.ux = fma(fma(m.rho, qx, nx), nr, qx);
+  m.uy = fma(fma(m.rho, qy, ny), nr, qy);
+  const float least =
+      fminf(fminf(fabsf(m.ux.x), fabsf(m.ux.y)), fminf(fabsf(m.uy.x), fabsf(m.uy.y)));
+  if (!(least >= kLeastQuotient)) {
+    if (needs_division(m.jx.x, m.ux.x) || needs_division(m.jx.y, m.ux.y) ||
+        needs_division(m.jy.x, m.uy.x) || needs_division(m.jy.y, m.uy.y)) {
+      m.ux = make_float2(__fdiv_rn(m.jx.x, m.rho.x), __fdiv_rn(m.jx.y, m.rho.y));
+      m.uy = make_float2(__fdiv_rn(m.jy.x, m.rho.x), __fdiv_rn(m.jy.y, m.rho.y));
+    }
+  }
   m.pxx = fma(nx, m.ux, fmas(-kCs2, m.drho, v.xx));
   m.pxy = fma(nx, m.uy, v.xy);
-  m.pyy = fma(muls(-1.0f, m.jy), m.uy, fmas(-kCs2, m.drho, v.yy));
+  m.pyy = fma(ny, m.uy, fmas(-kCs2, m.drho, v.yy));
   return m;
 }
 
-// Populations inside the chip: f_i times 2^(number of its non-zero velocity
-// components), which leaves the factors 1/2 out of the synthesis; the sums
-// put them back (powers of two change no rounding short of underflow).
+// mom3 of lbrr_device.cuh
 __device__ __forceinline__ void sum3(V a, V b, V c, V &s0, V &s1, V &s2) {
   s2 = add(a, c);
-  s0 = fmas(0.5f, s2, b);
+  s0 = add(s2, b);
   s1 = sub(c, a);
 }
 __device__ __forceinline__ Mom2 moments_of(const V (&f)[9]) {
   V s0[3], s1[3], s2[3], t0, t1, t2;
 #pragma unroll
   for (int l = 0; l < 3; ++l) sum3(f[3 * l], f[3 * l + 1], f[3 * l + 2], s0[l], s1[l], s2[l]);
-  V m01, m02, m10, m11, m20;
   Mom2 m;
-  sum3(s0[0], s0[1], s0[2], m.drho, m01, m02);
-  sum3(s1[0], s1[1], s1[2], m10, m11, t0);
-  sum3(s2[0], s2[1], s2[2], m20, t1, t2);
-  m.jx = muls(0.5f, m10);
-  m.jy = muls(0.5f, m01);
-  m.xx = muls(0.5f, m20);
-  m.xy = muls(0.25f, m11);
-  m.yy = muls(0.5f, m02);
+  sum3(s0[0], s0[1], s0[2], m.drho, m.jy, m.yy);
+  sum3(s1[0], s1[1], s1[2], m.jx, m.xy, t0);
+  sum3(s2[0], s2[1], s2[2], m.xx, t1, t2);
   return m;
 }
 
+// The outer two populations come out as twice their value. TWICE: so do the
+// coefficients come in; the factor 1/2 of coefficient 1 goes into the two sums it
+// enters, as the compiler has it in the single updates, and the others take it by
+// themselves, so that a value which underflows is rounded where theirs is.
+template <bool TWICE>
 __device__ __forceinline__ void synth3(V c0, V c1, V c2, V &om, V &oz, V &op) {
+  if (TWICE) c0 = muls(0.5f, c0), c2 = muls(0.5f, c2);
   const V q = fmas(kCs2, c0, c2);
   oz = sub(c0, q);
-  op = add(q, c1);
-  om = sub(q, c1);
+  op = TWICE ? fmas(0.5f, c1, q) : add(q, c1);
+  om = TWICE ? fmas(-0.5f, c1, q) : sub(q, c1);
 }
 __device__ __forceinline__ void post_collision(const Mac2 &m, float om1, V (&f)[9]) {
   const V uy = m.uy, uyy = mul(uy, uy), uxx = mul(m.ux, m.ux), ux2 = add(m.ux, m.ux);
@@ -107,14 +112,18 @@ __device__ __forceinline__ void post_collision(const Mac2 &m, float om1, V (&f)[
   c[2][1] = fma(uxx, q1_1, fma(ux2, pxy, mul(pxx, uy)));
   c[2][2] = fma(uxx, q1_2, fma(ux2, q3_2, mul(pxx, uyy)));
 #pragma unroll
-  for (int b = 0; b < 3; ++b) synth3(c[0][b], c[1][b], c[2][b], s[0][b], s[1][b], s[2][b]);
+  for (int b = 0; b < 3; ++b)
+    synth3<false>(c[0][b], c[1][b], c[2][b], s[0][b], s[1][b], s[2][b]);
+  synth3<true>(s[0][0], s[0][1], s[0][2], f[0], f[3], f[6]);
+  synth3<false>(s[1][0], s[1][1], s[1][2], f[1], f[4], f[7]);
+  synth3<true>(s[2][0], s[2][1], s[2][2], f[2], f[5], f[8]);
 #pragma unroll
-  for (int ix = 0; ix < 3; ++ix) synth3(s[ix][0], s[ix][1], s[ix][2], f[ix], f[ix + 3], f[ix + 6]);
+  for (int i = 0; i < 3; ++i) {
+    f[i] = muls(0.5f, f[i]);
+    f[i + 6] = muls(0.5f, f[i + 6]);
+  }
 }
 
-__host__ __device__ constexpr float scale2(int i) {
-  return (vel(i, 0) ? 2.0f : 1.0f) * (vel(i, 1) ? 2.0f : 1.0f);
-}
 __device__ __forceinline__ float &lane(V &v, int k) { return k ? v.y : v.x; }
 
 // ------------------------------------------------------------------ memory --
