@@ -146,8 +146,8 @@ LB_API int lb_init_fields(lb_ctx *ctx, const float *rho, const float *u, int ini
 /* Advance n >= 0 full collide-and-stream updates (eq_discr_bgk_reg). n == 0 is
  * a no-op. Asynchronous on the context's stream. Without a learned closure,
  * runs of updates of a periodic FP32 store go through the moments of the cells
- * where that is faster (scratch of up to a quarter of the free memory, kept by
- * the context; without it the updates run one by one), and other runs of 8
+ * where that is faster (through scratch, lb_set_run_limit; without it the updates
+ * run one by one), and other runs of 8
  * updates are replayed from a CUDA graph that the context captures
  * on first use (one per starting AA parity, on a stream of its own); the
  * results are those of update-by-update launches, bit for bit (while the
@@ -157,6 +157,23 @@ LB_API int lb_init_fields(lb_ctx *ctx, const float *rho, const float *u, int ini
  * update waits (boundedly) for its own bulk copies; if such a wait ever
  * expires, the next lb_diagnostics or lb_get_state returns LB_ETIMEOUT. */
 LB_API int lb_step(lb_ctx *ctx, int n);
+
+/* Scratch of runs of updates: 80 bytes a cell in 3D, 48 in 2D (rows rounded up to
+ * 32 cells). A context allocates it when lb_step first has a use for it, where it
+ * takes at most `bytes` (-1, the default: a quarter of the memory free then; 0:
+ * never), and keeps it until it is destroyed, until a lower limit is set here, or
+ * until an allocation of this library finds no other memory (any context gives
+ * its own back then, and looks again at its next run). What is freed waits for
+ * the work that uses it. */
+LB_API int lb_set_run_limit(lb_ctx *ctx, long long bytes);
+
+/* How the last lb_step of n > 0 went. */
+#define LB_RUN_SINGLE 0  /* update by update (singly, from a graph, with the closure) */
+#define LB_RUN_MOMENTS 1 /* 3D: on the moments */
+#define LB_RUN_TILES 2   /* 2D: on the moments, tiles in registers */
+#define LB_RUN_ROWS 3    /* 2D: on the moments, streaming rows */
+/* out[0..2]: that, the bytes of scratch held, the limit (-1: the default). */
+LB_API int lb_run_info(lb_ctx *ctx, long long *out);
 
 /* Macroscopic fields of the current populations into device buffers:
  * rho [N], u [D][N], pi1 [3 or 6][N] (xx, xy, yy in 2D; xx, xy, xz, yy, yz, zz

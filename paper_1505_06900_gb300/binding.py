@@ -17,6 +17,7 @@ _PKG = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_PKG, "_build", "liblbrr.so")
 
 LB_OK, LB_EINVAL, LB_ENOMEM, LB_ECUDA, LB_EDIVERGED, LB_ETIMEOUT = 0, 1, 2, 3, 4, 5
+RUN_SINGLE, RUN_MOMENTS, RUN_TILES, RUN_ROWS = 0, 1, 2, 3  # routes of a step(n)
 D2Q9, D3Q19, D3Q27 = 9, 19, 27
 STORE_F32, STORE_F16, STORE_BF16 = 0, 1, 2
 COLLIDE_RR, COLLIDE_REG2, COLLIDE_BGK = 0, 1, 2
@@ -33,6 +34,8 @@ SIGNATURES = {
     "lb_set_stream": (_i, [_vp, _vp]),
     "lb_init_fields": (_i, [_vp, _vp, _vp, _i]),
     "lb_step": (_i, [_vp, _i]),
+    "lb_set_run_limit": (_i, [_vp, _ll]),
+    "lb_run_info": (_i, [_vp, ctypes.POINTER(_ll)]),
     "lb_moments": (_i, [_vp, _vp, _vp, _vp]),
     "lb_diagnostics": (_i, [_vp, _vp]),
     "lb_enstrophy": (_i, [_vp, _vp]),
@@ -195,6 +198,17 @@ class Solver:
 
     def step(self, n: int = 1):
         self._check(self._lib.lb_step(self._h, int(n)))
+
+    def set_run_limit(self, max_bytes: int = -1):
+        """Most scratch that runs of updates may take and keep (-1: a quarter of the free
+        memory, 0: none, and what is held is freed)."""
+        self._check(self._lib.lb_set_run_limit(self._h, int(max_bytes)))
+
+    def run_info(self) -> dict:
+        """How the last step(n) went (RUN_*), the scratch held and its limit in bytes."""
+        out = (ctypes.c_longlong * 3)()
+        self._check(self._lib.lb_run_info(self._h, out))
+        return dict(zip(["route", "bytes", "limit"], list(out)))
 
     def moments(self):
         """(rho [nz,ny,nx], u [D,...], pi1 [3|6,...]) as CUDA tensors."""

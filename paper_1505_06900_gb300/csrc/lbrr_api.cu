@@ -5,6 +5,7 @@
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
+#include <mutex>
 #include <new>
 
 #include <nvtx3/nvToolsExt.h>
@@ -23,9 +24,14 @@ struct lb_ctx {
   int device = 0;
   size_t elem = 4;         // bytes per stored population
   void *f = nullptr;       // population store, q * n elements
-  void *run = nullptr;     // scratch of the kernels for runs of updates, allocated on first
-                           // use; between calls the state is always in f
-  bool run_off = false;    // it does not fit: update by update
+  // Scratch of the kernels for runs of updates; between calls the state is always
+  // in f, so that another context that is out of memory may free it (run_mutex).
+  std::mutex run_mutex;
+  void *run = nullptr;
+  long long run_bytes = 0;   // its size
+  long long run_limit = -1;  // most it may take (-1: a quarter of the free memory)
+  int route = LB_RUN_SINGLE;  // of the last lb_step
+  lb_ctx *next = nullptr;    // in the list of contexts
   lbrr::Run2Plans run2;    // D2Q9: the tiles of a run's passes, set on first use
   int sms = 0;                 // SMs of the device
   int red_blocks = 0;          // partial-sum blocks: kRedBlocksPerSm x the device's SMs
@@ -135,6 +141,56 @@ int need_device(lb_ctx *c, const void *p, const char *what) {
     if (rc_ != LB_OK) return rc_;              \
   } while (0)
 
+// Allocations and releases must not disturb a stream capture that another thread
+// or stream has under way.
+struct RelaxedCapture {
+  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+  RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+  ~RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+};
+
+// Every context, for the scratch that they can do without.
+std::mutex g_contexts_mutex;
+lb_ctx *g_contexts = nullptr;
+
+// Gives back a context's scratch for runs (run_mutex held; cudaFree waits for the
+// kernels that use it).
+void free_run(lb_ctx *c) {
+  if (!c->run) return;
+  RelaxedCapture relaxed;
+  cudaFree(c->run);
+  c->run = nullptr;
+  c->run_bytes = 0;
+}
+
+// Gives back what the contexts of a device hold for runs of updates; false if
+// none holds any.
+bool free_runs(int device) {
+  bool any = false;
+  std::lock_guard<std::mutex> list(g_contexts_mutex);
+  for (lb_ctx *c = g_contexts; c; c = c->next) {
+    if (c->device != device) continue;
+    std::lock_guard<std::mutex> lock(c->run_mutex);
+    any = any || c->run;
+    free_run(c);
+  }
+  return any;
+}
+
+// cudaMalloc on the current device, at the cost of the scratch for runs where
+// there is no other memory left.
+template <typename T>
+cudaError_t device_malloc(T **p, size_t bytes) {
+  *p = nullptr;
+  cudaError_t e = cudaMalloc(p, bytes);
+  int device = 0;
+  if (e != cudaErrorMemoryAllocation || cudaGetDevice(&device) != cudaSuccess ||
+      !free_runs(device))
+    return e;
+  cudaGetLastError();
+  return cudaMalloc(p, bytes);
+}
+
 int free_all(lb_ctx *c) {
   for (auto &ge : c->graph)
     if (ge) cudaGraphExecDestroy(ge);
@@ -142,8 +198,7 @@ int free_all(lb_ctx *c) {
   if (c->capture) cudaStreamDestroy(c->capture);
   c->capture = nullptr;
   if (c->f) cudaFree(c->f);
-  if (c->run) cudaFree(c->run);
-  c->run = nullptr;
+  free_run(c);
   if (c->partials) cudaFree(c->partials);
   if (c->dout) cudaFree(c->dout);
   if (c->status) cudaFree(c->status);
@@ -166,7 +221,7 @@ int free_all(lb_ctx *c) {
 
 int ensure_fields(lb_ctx *c) {
   if (c->fields) return LB_OK;
-  cudaError_t e = cudaMalloc(&c->fields, sizeof(float) * (size_t)(1 + c->d) * (size_t)c->g.n);
+  cudaError_t e = device_malloc(&c->fields, sizeof(float) * (size_t)(1 + c->d) * (size_t)c->g.n);
   if (e != cudaSuccess) {
     c->fields = nullptr;
     cudaGetLastError();
@@ -272,11 +327,11 @@ int lb_create_ex(lb_ctx **out, const lb_options *opt) {
   c->sms = sms;
   c->red_blocks = lbrr::kRedBlocksPerSm * sms;
   const size_t bytes = c->elem * (size_t)c->q * (size_t)n;
-  e = cudaMalloc(&c->f, bytes);
+  e = device_malloc(&c->f, bytes);
   if (e == cudaSuccess)
-    e = cudaMalloc(&c->partials, sizeof(double) * (size_t)c->red_blocks * lbrr::kRedValues);
-  if (e == cudaSuccess) e = cudaMalloc(&c->dout, sizeof(double) * lbrr::kRedValues);
-  if (e == cudaSuccess) e = cudaMalloc(&c->status, 2 * sizeof(int));
+    e = device_malloc(&c->partials, sizeof(double) * (size_t)c->red_blocks * lbrr::kRedValues);
+  if (e == cudaSuccess) e = device_malloc(&c->dout, sizeof(double) * lbrr::kRedValues);
+  if (e == cudaSuccess) e = device_malloc(&c->status, 2 * sizeof(int));
   if (e != cudaSuccess) {
     cudaGetLastError();
     free_all(c);
@@ -292,6 +347,11 @@ int lb_create_ex(lb_ctx **out, const lb_options *opt) {
     delete c;
     return fail(nullptr, LB_ECUDA, "initial clear failed: %s", cudaGetErrorString(e));
   }
+  {
+    std::lock_guard<std::mutex> list(g_contexts_mutex);
+    c->next = g_contexts;
+    g_contexts = c;
+  }
   *out = c;
   return LB_OK;
 }
@@ -304,6 +364,14 @@ int lb_create(lb_ctx **out, int lattice, int nx, int ny, int nz, double tau, int
 void lb_destroy(lb_ctx *c) {
   if (!c) return;
   DeviceGuard dg(c->device);
+  {
+    std::lock_guard<std::mutex> list(g_contexts_mutex);
+    for (lb_ctx **p = &g_contexts; *p; p = &(*p)->next)
+      if (*p == c) {
+        *p = c->next;
+        break;
+      }
+  }
   if (c->stream) cudaStreamSynchronize(c->stream);
   free_all(c);
   delete c;
@@ -368,24 +436,47 @@ cudaGraphExec_t step_graph(lb_ctx *c, float om1) {
   return c->graph[p];
 }
 
-// The scratch for runs of updates, allocated on first use where it takes at
-// most a quarter of the device's free memory (the context works without it,
-// one update at a time). The allocation must not disturb a stream capture
-// that another thread or stream has under way.
+// The scratch for runs of updates (run_mutex held), allocated when a run first
+// finds it within the limit: the context works without it, one update at a time.
 bool ensure_run(lb_ctx *c, size_t bytes) {
-  if (c->run || c->run_off) return c->run != nullptr;
-  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
-  cudaThreadExchangeStreamCaptureMode(&mode);
-  size_t free_b = 0, total_b = 0;
-  cudaError_t e = cudaMemGetInfo(&free_b, &total_b);
-  if (e == cudaSuccess && bytes <= free_b / 4) e = cudaMalloc(&c->run, bytes);
-  cudaThreadExchangeStreamCaptureMode(&mode);
+  if (c->run) return true;
+  RelaxedCapture relaxed;
+  size_t most = (size_t)c->run_limit, total = 0;
+  cudaError_t e = cudaSuccess;
+  if (c->run_limit < 0) {
+    e = cudaMemGetInfo(&most, &total);
+    most /= 4;
+  }
+  if (e == cudaSuccess && bytes <= most) e = cudaMalloc(&c->run, bytes);
   if (e != cudaSuccess) {
     cudaGetLastError();
     c->run = nullptr;
   }
-  c->run_off = !c->run;
+  if (c->run) c->run_bytes = (long long)bytes;
   return c->run != nullptr;
+}
+
+// The n updates of lb_step as a run on the moments; false where the updates go
+// one by one.
+bool step_run(lb_ctx *c, int n, float om1, cudaError_t *e) {
+  const bool flat = c->q == 9;
+  if (flat ? !lbrr::moment_run2_supported(c->q, c->storage, c->collision, c->g, n)
+           : !lbrr::moment_run_supported(c->q, c->storage, c->collision, c->g, n, c->sms))
+    return false;
+  std::lock_guard<std::mutex> lock(c->run_mutex);
+  if (!ensure_run(c, flat ? lbrr::moment_run2_bytes(c->g) : lbrr::moment_run_bytes(c->g)))
+    return false;
+  if (flat) {
+    if (!c->run2.ready) lbrr::plan_moment_run2(c->g, c->sms, &c->run2);
+    bool rows = false;
+    *e = lbrr::launch_moment_run2(c->f, c->run, c->g, om1, c->parity, n, c->run2, &rows, c->stream);
+    c->route = rows ? LB_RUN_ROWS : LB_RUN_TILES;
+  } else {
+    *e = lbrr::launch_moment_run(c->q, c->collision, c->f, c->run, c->g, om1, c->parity, n, c->sms,
+                                 c->stream);
+    c->route = LB_RUN_MOMENTS;
+  }
+  return true;
 }
 
 }  // namespace
@@ -403,23 +494,10 @@ int lb_step(lb_ctx *c, int n) {
   const bool capturing = cudaStreamIsCapturing(c->stream, &cs) != cudaSuccess ||
                          cs != cudaStreamCaptureStatusNone;
   if (capturing) cudaGetLastError();
-  if (!c->closure && !capturing &&
-      lbrr::moment_run_supported(c->q, c->storage, c->collision, c->g, n, c->sms) &&
-      ensure_run(c, lbrr::moment_run_bytes(c->g))) {
-    cudaError_t e = lbrr::launch_moment_run(c->q, c->collision, c->f, c->run, c->g, om1, c->parity,
-                                            n, c->sms, c->stream);
-    if (e != cudaSuccess) return cuda_fail(c, e, "step launch");
-    c->parity = (c->parity + n) & 1;
-    c->steps += n;
-    return LB_OK;
-  }
-  if (!c->closure && !capturing &&
-      lbrr::moment_run2_supported(c->q, c->storage, c->collision, c->g, n) &&
-      ensure_run(c, lbrr::moment_run2_bytes(c->g))) {
-    if (!c->run2.ready) lbrr::plan_moment_run2(c->g, c->sms, &c->run2);
-    cudaError_t e = lbrr::launch_moment_run2(c->f, c->run, c->g, om1, c->parity, n, c->run2,
-                                             c->stream);
-    if (e != cudaSuccess) return cuda_fail(c, e, "step launch");
+  cudaError_t re = cudaSuccess;
+  if (n > 0) c->route = LB_RUN_SINGLE;
+  if (!c->closure && !capturing && step_run(c, n, om1, &re)) {
+    if (re != cudaSuccess) return cuda_fail(c, re, "step launch");
     c->parity = (c->parity + n) & 1;
     c->steps += n;
     return LB_OK;
@@ -460,6 +538,25 @@ int lb_step(lb_ctx *c, int n) {
     c->parity ^= 1;
     ++c->steps;
   }
+  return LB_OK;
+}
+
+int lb_set_run_limit(lb_ctx *c, long long bytes) {
+  LB_CHECK_CTX(c);
+  DeviceGuard dg(c->device);
+  std::lock_guard<std::mutex> lock(c->run_mutex);
+  c->run_limit = bytes < 0 ? -1 : bytes;
+  if (bytes >= 0 && c->run_bytes > bytes) free_run(c);
+  return LB_OK;
+}
+
+int lb_run_info(lb_ctx *c, long long *out) {
+  LB_CHECK_CTX(c);
+  if (!out) return fail(c, LB_EINVAL, "null output");
+  std::lock_guard<std::mutex> lock(c->run_mutex);
+  out[0] = c->route;
+  out[1] = c->run_bytes;
+  out[2] = c->run_limit;
   return LB_OK;
 }
 
@@ -665,15 +762,15 @@ int lb_mlp_create(lb_mlp **out) {
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, m->device);
   m->nblocks = sms > 0 ? sms : 1;
   const size_t P = lbrr::kMlpParams;
-  e = cudaMalloc(&m->d.params, 4 * P);
-  if (e == cudaSuccess) e = cudaMalloc(&m->d.adam_m, 4 * P);
-  if (e == cudaSuccess) e = cudaMalloc(&m->d.adam_v, 4 * P);
-  if (e == cudaSuccess) e = cudaMalloc(&m->d.w1, lbrr::kMlpWeightBytes);
-  if (e == cudaSuccess) e = cudaMalloc(&m->scaling, 4 * 37);
-  if (e == cudaSuccess) e = cudaMalloc(&m->gpart, 4 * P * (size_t)m->nblocks);
-  if (e == cudaSuccess) e = cudaMalloc(&m->lpart, 4 * (size_t)m->nblocks);
-  if (e == cudaSuccess) e = cudaMalloc(&m->dloss, sizeof(double));
-  if (e == cudaSuccess) e = cudaMalloc(&m->status, 2 * sizeof(int));
+  e = device_malloc(&m->d.params, 4 * P);
+  if (e == cudaSuccess) e = device_malloc(&m->d.adam_m, 4 * P);
+  if (e == cudaSuccess) e = device_malloc(&m->d.adam_v, 4 * P);
+  if (e == cudaSuccess) e = device_malloc(&m->d.w1, lbrr::kMlpWeightBytes);
+  if (e == cudaSuccess) e = device_malloc(&m->scaling, 4 * 37);
+  if (e == cudaSuccess) e = device_malloc(&m->gpart, 4 * P * (size_t)m->nblocks);
+  if (e == cudaSuccess) e = device_malloc(&m->lpart, 4 * (size_t)m->nblocks);
+  if (e == cudaSuccess) e = device_malloc(&m->dloss, sizeof(double));
+  if (e == cudaSuccess) e = device_malloc(&m->status, 2 * sizeof(int));
   if (e == cudaSuccess) e = cudaMemset(m->status, 0, 2 * sizeof(int));
   if (e != cudaSuccess) {
     cudaGetLastError();
@@ -867,11 +964,11 @@ static cudaError_t zero_now(void *p, size_t bytes) {
 static int ensure_mom(lb_ctx *c, bool for_step) {
   const bool conv = for_step && lbrr::mlp_conv_supported(c->g);
   cudaError_t e = cudaSuccess;
-  if (!conv && !c->mom) e = cudaMalloc(&c->mom, sizeof(float) * 10 * (size_t)c->g.n);
+  if (!conv && !c->mom) e = device_malloc(&c->mom, sizeof(float) * 10 * (size_t)c->g.n);
   if (e == cudaSuccess && for_step && !conv && !c->ystd)
-    e = cudaMalloc(&c->ystd, sizeof(float) * 17 * (size_t)c->g.n);
+    e = device_malloc(&c->ystd, sizeof(float) * 17 * (size_t)c->g.n);
   if (e == cudaSuccess && conv && !c->xs) {
-    e = cudaMalloc(&c->xs, lbrr::feature_source_bytes(c->g));
+    e = device_malloc(&c->xs, lbrr::feature_source_bytes(c->g));
     if (e == cudaSuccess) {
       // for the row padding beyond the halo, which no update writes: rows of whole
       // tiles only copy it, other grids multiply it into tile rows that are dropped
@@ -996,7 +1093,7 @@ int lb_set_closure_ex(lb_ctx *c, const lb_mlp *m, float bound, float dead_zone) 
   rc = ensure_mom(c, true);
   if (rc != LB_OK) return rc;
   if (!c->fallbacks) {
-    cudaError_t e = cudaMalloc(&c->fallbacks, sizeof(unsigned long long));
+    cudaError_t e = device_malloc(&c->fallbacks, sizeof(unsigned long long));
     if (e == cudaSuccess) e = zero_now(c->fallbacks, sizeof(unsigned long long));
     if (e != cudaSuccess) {
       cudaGetLastError();

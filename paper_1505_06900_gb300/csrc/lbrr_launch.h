@@ -54,8 +54,9 @@ cudaError_t launch_march(int kind, float *f, const float *a, float *b, const Gri
 bool moment_run2_supported(int q, int storage, int model, const Grid &g, int steps);
 size_t moment_run2_bytes(const Grid &g);
 void plan_moment_run2(const Grid &g, int sms, Run2Plans *plans);
-cudaError_t launch_moment_run2(void *f, void *scratch, const Grid &g, float om1,
-                               int parity, int steps, const Run2Plans &plans, cudaStream_t st);
+// *rows: whether the row-streaming kernel was taken.
+cudaError_t launch_moment_run2(void *f, void *scratch, const Grid &g, float om1, int parity,
+                               int steps, const Run2Plans &plans, bool *rows, cudaStream_t st);
 
 // The one-thread-per-cell kernel of launch_step (lbrr_step.cu), for any grid
 // without walls and any storage.

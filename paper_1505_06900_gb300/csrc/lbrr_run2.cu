@@ -260,7 +260,7 @@ void plan_moment_run2(const Grid &g, int sms, Run2Plans *plans) {
 }
 
 cudaError_t launch_moment_run2(void *f, void *scratch, const Grid &g, float om1, int parity,
-                               int steps, const Run2Plans &plans, cudaStream_t st) {
+                               int steps, const Run2Plans &plans, bool *rows, cudaStream_t st) {
   float *s = static_cast<float *>(f), *m0 = static_cast<float *>(scratch);
   float *m1 = m0 + 192 * (size_t)blocks2_x(g) * (size_t)g.ny;
   // updates a pass: the cheapest by the estimate, shared out evenly; the last
@@ -283,6 +283,7 @@ cudaError_t launch_moment_run2(void *f, void *scratch, const Grid &g, float om1,
       }
     }
   }
+  *rows = march;
   if (cost < 0) return cudaErrorInvalidValue;
   int done = 0;
   for (int k = 0; k < passes; ++k) {
