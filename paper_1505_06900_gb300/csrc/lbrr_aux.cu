@@ -262,7 +262,7 @@ __global__ void __launch_bounds__(kRedThreads)
 // leaves less, or whose square would leave the range where its low part is an
 // FP32 number, and the nodes on walls, take FP64. With a cell to a thread that took 227 us, waiting for
 // twelve scalar loads; with four cells of a row, which the float4 rows of
-// nx % 4 == 0 allow, 106 us.
+// nx % 4 == 0 allow, 120 us.
 constexpr int kCurlFlush = 64;
 // The roundings that the transformations count on are asked for by name: a
 // product fused into the sum that follows would bring in its low part twice.

@@ -6,8 +6,9 @@
 // the chain. Data read after the wait is read with ordinary loads or
 // asynchronous copies, not as read-only for the length of the kernel (no
 // const __restrict__ parameters for it). Launch and start-up of a short kernel
-// then cost nothing: 50 D2Q9 updates of 128^2 cells and their read-back 61.5 -> 48.1 us, a
-// training step of 8192 rows 18.5 -> 13.9, a closure step of 64^3 38.6 -> 33.9.
+// then cost nothing: 50 D2Q9 updates of 128^2 cells and their read-back 61.5 ->
+// 48.1 us (50.2 as the runs are now), a training step of 8192 rows 18.5 -> 13.9, a
+// closure step of 64^3 38.6 -> 33.9.
 #pragma once
 
 #include <cuda_runtime.h>

@@ -2,8 +2,9 @@
 // wall kernel for bounded grids; for 16-bit stores the direct paired kernel
 // for the even update and the staged row-segment kernel for the odd one where
 // the row length allows, else the whole-row kernel, else two cells per thread;
-// otherwise (and for FP32 stores) one thread per cell. Kept apart from the kernels so that a change of
-// routing leaves their sources, and the profiles keyed to them, unchanged.
+// otherwise (and for FP32 stores) one thread per cell. Kept apart from the
+// kernels so that a change of routing leaves their sources, and the profiles
+// keyed to them, unchanged.
 #include "lbrr_launch.h"
 
 namespace lbrr {

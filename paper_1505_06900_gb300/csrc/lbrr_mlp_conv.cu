@@ -248,7 +248,8 @@ __global__ void __launch_bounds__(kConvThreads, 1)
         nb = k < 6 ? (k >> 1) + 3 * r9 : -1;
         ch = 8 + (k & 1);
       }
-      w[k] = nb >= 0 ? __bfloat16_as_ushort(p.w1[cm_offset(n, kMlpMoments * nb + ch, kMlpIn) / 2]) : 0;
+      w[k] = nb < 0 ? 0
+                    : __bfloat16_as_ushort(p.w1[cm_offset(n, kMlpMoments * nb + ch, kMlpIn) / 2]);
     }
     if (kind == 1 && h == 1 && r9 == 4) {  // b1 = b_hi + b_lo on the constant inputs
       const __nv_bfloat16 hi = __float2bfloat16_rn(p.b1[n]);
@@ -618,8 +619,8 @@ PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder() {
   static const PFN_cuTensorMapEncodeTiled_v12000 encode = [] {
     cudaDriverEntryPointQueryResult q;
     void *fn = nullptr;
-    const cudaError_t e =
-        cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000, cudaEnableDefault, &q);
+    const cudaError_t e = cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000,
+                                                           cudaEnableDefault, &q);
     if (e != cudaSuccess || q != cudaDriverEntryPointSuccess) fn = nullptr;
     return reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(fn);
   }();

@@ -10,9 +10,9 @@
 // bytes apart (leading byte offset) and adjacent 8-row groups K/8 * 128 bytes
 // apart (stride byte offset), as they lie in memory. A tile's 128 input rows
 // come by TMA in boxes of 64 columns in the layout with 128-byte swizzle, the
-// last 32 with 64-byte swizzle; one thread of the group issues the MMAs of a layer (M = 128, N = 64, 64, 32)
-// and commits them to the group's mbarrier; the threads, two to a row (TMEM
-// lane), then read the accumulator (tcgen05.ld 32x32b), add the bias, apply
+// last 32 with 64-byte swizzle; one thread of the group issues the MMAs of a
+// layer (M = 128, N = 64, 64, 32) and commits them to the group's mbarrier; the
+// threads, two to a row (TMEM lane), then read the accumulator (tcgen05.ld 32x32b), add the bias, apply
 // tanh and write the BF16 row back into TMEM (tcgen05.st), the A operand of the
 // next layer.
 //
@@ -101,7 +101,8 @@ __device__ __forceinline__ void hidden_epilogue(uint32_t taddr, const float *bia
     if (TRACE && hrow)
 #pragma unroll
       for (int k = 0; k < 16; k += 4)
-        *reinterpret_cast<float4 *>(hrow + c0 + k) = make_float4(v[k], v[k + 1], v[k + 2], v[k + 3]);
+        *reinterpret_cast<float4 *>(hrow + c0 + k) =
+            make_float4(v[k], v[k + 1], v[k + 2], v[k + 3]);
 #pragma unroll
     for (int k = 0; k < 16; k += 2) q[8 * i + k / 2] = pack2(v[k], v[k + 1]);
   }
@@ -143,8 +144,8 @@ __device__ __forceinline__ void features_gather(const MlpDevice &p, const float 
 template <bool FROM_MOM, bool TRACE = false>
 __global__ void __launch_bounds__(kTcThreads, 1)
     mlp_tc_kernel(MlpDevice p, const __grid_constant__ CUtensorMap x_map,
-                  const __grid_constant__ CUtensorMap x_last, const float *__restrict__ mom, const Grid g, long long M,
-                  float *__restrict__ Y, int *status, float *__restrict__ H) {
+                  const __grid_constant__ CUtensorMap x_last, const float *__restrict__ mom,
+                  const Grid g, long long M, float *__restrict__ Y, int *status, float *__restrict__ H) {
   extern __shared__ __align__(1024) unsigned char smem[];
   const int tid = threadIdx.x, warp = tid >> 5;
   const int gr = tid / kGroupThreads, gt = tid % kGroupThreads;
